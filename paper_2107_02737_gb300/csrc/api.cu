@@ -162,8 +162,8 @@ struct Carver {
 // reads a compact set of row and column panels and the operand matrices, which
 // are larger than L2, are fetched from HBM about once per run.
 void build_tiles_uncached(int path, int np, int cg, std::vector<int2> &t) {
-    const int bm = (path == PATH_SIMT) ? SIMT_T : TC_BM * cg;
-    const int bn = (path == PATH_SIMT) ? SIMT_T : TC_BN;
+    const int bm = (path == PATH_SIMT) ? simt_tile_side(np) : TC_BM * cg;
+    const int bn = (path == PATH_SIMT) ? simt_tile_side(np) : TC_BN;
     const int nbi = (np + bm - 1) / bm, nbj = (np + bn - 1) / bn;  // a last pair tile may overhang np
     const int sbi = 2048 / bm, sbj = 2048 / bn;  // tiles per super-block side
     std::vector<std::pair<long long, int2>> keyed;
@@ -195,8 +195,8 @@ void build_tiles(int path, int np, int cg, std::vector<int2> &t) {
 
 // Number of tiles of the table above, counted without building it.
 int ntiles_for(int path, int np, int cg) {
-    const int bm = (path == PATH_SIMT) ? SIMT_T : TC_BM * cg;
-    const int bn = (path == PATH_SIMT) ? SIMT_T : TC_BN;
+    const int bm = (path == PATH_SIMT) ? simt_tile_side(np) : TC_BM * cg;
+    const int bn = (path == PATH_SIMT) ? simt_tile_side(np) : TC_BN;
     const int nbi = (np + bm - 1) / bm, nbj = (np + bn - 1) / bn;
     int count = 0;
     for (int bj = 0; bj < nbj; ++bj) count += std::min(nbi, ((bj + 1) * bn + bm - 1) / bm);
@@ -213,6 +213,7 @@ struct Plan {
     int mode, path, precision;
     bool dataflow = false;            // see flow_eligible
     int cg = 1;                       // CTAs per tensor-core tile
+    int simt_tmax = 128;              // FP32 path: largest tile side of the instances
     std::vector<InstSpec> inst;       // non-trivial instances, in launch order
     std::vector<int> slots;           // nslots_x per instance
     std::vector<int> ckpt_s, ckpt_k;  // adjoint checkpoint stride and kept layers (0: every layer kept)
@@ -414,7 +415,7 @@ struct LaunchGeometry {
     bool known = false;
     DeviceInfo di;
     int grid_cg[3] = {0, 0, 0};
-    int simt_per_sm = 0;
+    int simt_per_sm[3] = {0, 0, 0};   // resident CTAs per SM with tiles up to 32, 64, 128
 };
 bool launch_geometry(LaunchGeometry &g) {
     static std::mutex mu;
@@ -433,7 +434,7 @@ bool launch_geometry(LaunchGeometry &g) {
         if (e.di.major == 10 && e.di.minor == 3) {
             e.grid_cg[2] = tc_grid_size(2, e.di.sm);
             e.grid_cg[1] = tc_grid_size(1, e.di.sm);
-            e.simt_per_sm = simt_blocks_per_sm();
+            for (int k = 0; k < 3; ++k) e.simt_per_sm[k] = simt_blocks_per_sm(32 << k);
         }
         e.known = true;
     }
@@ -460,9 +461,13 @@ sp2_status choose_launch(Plan &pl, int want, int &grid) {
         }
         if (grid <= 0) return SP2_ERR_UNSUPPORTED;
     } else {
-        const int per_sm = geo.simt_per_sm;
+        pl.simt_tmax = simt_tile_side(pl.max_np);
+        const int per_sm = geo.simt_per_sm[pl.simt_tmax == 32 ? 0 : pl.simt_tmax == 64 ? 1 : 2];
         if (per_sm <= 0) return SP2_ERR_UNSUPPORTED;
-        grid = per_sm * di.sm;
+        // No more CTAs than a round has tiles: the grid barrier costs less.
+        int tiles = 0;
+        for (auto &sp : pl.inst) tiles += ntiles_for(PATH_SIMT, round_up(sp.n, PAD), 1);
+        grid = std::max(1, std::min(per_sm * di.sm, tiles));
     }
     return SP2_OK;
 }
@@ -551,6 +556,7 @@ sp2_status prepare(Prepared &P, const sp2_opts &o, double tol, void *ws, size_t 
         d.nslots_x = pl.slots[i];
         d.part_cap = std::max(d.parts, initb);
         d.fin_blocks = P.fin_blocks;
+        d.simt_t = (pl.path == PATH_SIMT) ? simt_tile_side(np) : 0;
         d.ctl = d_ctl + i;
         d.part[0] = (Part *)c.take(sizeof(Part) * d.part_cap);
         d.part[1] = (Part *)c.take(sizeof(Part) * d.part_cap);
@@ -770,7 +776,7 @@ sp2_status enqueue(const Prepared &P, cudaStream_t s, cudaEvent_t *ev, bool fres
         rp.blk_src = P.d_blk_src;
     }
     if (ev) CK(cudaEventRecord(ev[1], s));
-    CK(pl.path == PATH_TC ? launch_tc_persistent(rp, pl.cg, P.grid, s) : launch_simt_persistent(rp, P.grid, s));
+    CK(pl.path == PATH_TC ? launch_tc_persistent(rp, pl.cg, P.grid, s) : launch_simt_persistent(rp, pl.simt_tmax, P.grid, s));
     if (ev) CK(cudaEventRecord(ev[2], s));
     CK(launch_finalize(P.d_inst, B, P.fin_blocks, pl.mode == MODE_APPLY ? MODE_DENSITY : pl.mode, s));
     if (ev) CK(cudaEventRecord(ev[3], s));

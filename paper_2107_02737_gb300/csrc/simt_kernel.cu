@@ -1,7 +1,7 @@
 // simt_kernel.cu -- the FP32 CUDA-core SP2 chain (the plain-precision comparator).
 //
 // One cooperative persistent launch runs every layer: per round each CTA takes
-// upper-triangle 128 x 128 tiles (bi <= bj) of X_{n+1} = X_n^2 or 2 X_n - X_n^2
+// upper-triangle T x T tiles (bi <= bj; T = 32, 64 or 128 by size) of X_{n+1} = X_n^2 or 2 X_n - X_n^2
 // (or the accelerated layer), computes the tile's product with FP32 FMAs on the
 // centred operand X - I/2 (the B operand is rows of X because X is symmetric),
 // writes the tile and its mirror, and records FP64 partials of
@@ -13,69 +13,137 @@ namespace sp2i {
 
 namespace {
 
-constexpr int BK = 16;
-constexpr int LDS = SIMT_T + 4;  // padded smem row (floats), keeps float4 alignment
 
+// Tile side T with 128 threads as 8 (rows) x 16 (columns): a thread owns TM x TN
+// elements, rows in groups of four 32 apart, columns in groups of CW 16 CW apart.
+// What bounds the inner loop is shared-memory reads: a warp's read of one float per
+// lane costs a cycle of the SM's port, TM + TN of them per TM x TN FMAs (and those
+// TM TN / 4 cycles of the four FMA pipes).  16 x 8 elements per thread (24 cycles
+// against 32) left room that 8 x 8 (16 against 16) did not, packed FMAs free the issue
+// slots for it, and fragments read one k ahead hide its latency with one or two warps
+// per scheduler: N = 3000 from 651 to 525 us per layer (58 to 72 % of the FP32 peak at
+// 1.92 GHz over the executed tiles).
+template <int T>
+struct SimtCfg {
+    static constexpr int BK = (T == 128) ? 8 : 16;      // K elements per staged block
+    static constexpr int TM = T / 8, TN = T / 16;       // 16 x 8, 8 x 4, 4 x 2
+    static constexpr int CW = TN < 4 ? TN : 4;          // adjacent columns per thread
+    static constexpr int LDS = T + 4;                   // padded smem row (floats), keeps 16-byte alignment
+    static constexpr int KPT = BK * T / SIMT_THREADS;   // K elements of one row a thread stages: 16, 8, 4
+    static constexpr int FLOATS = 2 * 2 * BK * LDS;     // A and B, double-buffered
+};
+
+template <int TMAX>
 struct SimtSmem {
-    float A[2][BK][LDS];
-    float B[2][BK][LDS];
+    float stage[SimtCfg<TMAX>::FLOATS];
     double red[SIMT_THREADS / 32][2];
 };
-static_assert(sizeof(float) * 2 * BK * LDS >= 4 * MAX_BATCH * sizeof(double) + 4 * (SIMT_THREADS / 32) * sizeof(double),
-              "round sums reuse the A staging buffers");
+
+// Two FP32 FMAs in one instruction (each rounded as a scalar FMA): acc = a b + acc.
+__device__ __forceinline__ void ffma2(unsigned long long &acc, unsigned long long a, unsigned long long b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
 
 // acc = Y^2 over the tile for the centred operand Y = X - I/2 (I on the n real
 // diagonal entries): Y has the eigenvalues of X shifted into [-1/2, 1/2], so the
-// FP32 sums run over smaller terms; the epilogue adds X - I/4 back.
-__device__ __forceinline__ void simt_tile_mma(const float *__restrict__ X, int np, int n, int r0, int c0,
-                                              SimtSmem &sm, float acc[8][8]) {
+// FP32 sums run over smaller terms; the epilogue adds X - I/4 back.  Every element is
+// one chain of FMAs over increasing k, whatever T is.
+template <int T>
+__device__ __forceinline__ void simt_tile_mma(const float *X, int np, int n, int r0, int c0, float *stage,
+                                              unsigned long long (&acc)[SimtCfg<T>::TM / 2][SimtCfg<T>::TN]) {
+    using C = SimtCfg<T>;
+    constexpr int BK = C::BK;
     const int tid = threadIdx.x;
     const int tx = tid & 15, ty = tid >> 4;
-    const int lrow = tid >> 1, lk = (tid & 1) * 8;
+    // Staging: consecutive threads take consecutive rows, so the transposed stores
+    // are free of bank conflicts.
+    const int lrow = tid % T, lk = (tid / T) * C::KPT;
     const float *Ap = X + (size_t)(r0 + lrow) * np + lk;
     const float *Bp = X + (size_t)(c0 + lrow) * np + lk;
+    float *const sA = stage, *const sB = stage + 2 * BK * C::LDS;
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+    for (int i = 0; i < C::TM / 2; ++i)
 #pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = 0.0f;
+        for (int j = 0; j < C::TN; ++j) acc[i][j] = 0ull;
 
-    float4 ra0 = *(const float4 *)Ap, ra1 = *(const float4 *)(Ap + 4);
-    float4 rb0 = *(const float4 *)Bp, rb1 = *(const float4 *)(Bp + 4);
-    auto stash = [&](int buf, int kt) {
-        const float a[8] = {ra0.x, ra0.y, ra0.z, ra0.w, ra1.x, ra1.y, ra1.z, ra1.w};
-        const float b[8] = {rb0.x, rb0.y, rb0.z, rb0.w, rb1.x, rb1.y, rb1.z, rb1.w};
-        const int k0 = kt * BK + lk;
+    float4 ra[C::KPT / 4], rb[C::KPT / 4];
+    auto fetch = [&](int kt) {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int k = k0 + q;
-            sm.A[buf][lk + q][lrow] = (k == r0 + lrow && k < n) ? a[q] - 0.5f : a[q];
-            sm.B[buf][lk + q][lrow] = (k == c0 + lrow && k < n) ? b[q] - 0.5f : b[q];
+        for (int q = 0; q < C::KPT / 4; ++q) {
+            ra[q] = *(const float4 *)(Ap + (size_t)kt * BK + 4 * q);
+            rb[q] = *(const float4 *)(Bp + (size_t)kt * BK + 4 * q);
         }
     };
+    auto stash = [&](int buf, int kt) {
+        float *a = sA + (buf * BK + lk) * C::LDS + lrow, *b = sB + (buf * BK + lk) * C::LDS + lrow;
+        const int ka = r0 + lrow - kt * BK - lk, kb = c0 + lrow - kt * BK - lk;   // the diagonal's place, if in reach
+        const float ha = (r0 + lrow < n) ? 0.5f : 0.0f, hb = (c0 + lrow < n) ? 0.5f : 0.0f;
+#pragma unroll
+        for (int q = 0; q < C::KPT / 4; ++q) {
+            const float va[4] = {ra[q].x, ra[q].y, ra[q].z, ra[q].w};
+            const float vb[4] = {rb[q].x, rb[q].y, rb[q].z, rb[q].w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int k = 4 * q + e;
+                a[k * C::LDS] = (k == ka) ? va[e] - ha : va[e];
+                b[k * C::LDS] = (k == kb) ? vb[e] - hb : vb[e];
+            }
+        }
+    };
+    fetch(0);
     stash(0, 0);
     __syncthreads();
     const int nk = np / BK;
+#pragma unroll 1
     for (int kt = 0; kt < nk; ++kt) {
         const int buf = kt & 1;
-        if (kt + 1 < nk) {
-            const float *a = Ap + (size_t)(kt + 1) * BK, *b = Bp + (size_t)(kt + 1) * BK;
-            ra0 = *(const float4 *)a;
-            ra1 = *(const float4 *)(a + 4);
-            rb0 = *(const float4 *)b;
-            rb1 = *(const float4 *)(b + 4);
-        }
+        if (kt + 1 < nk) fetch(kt + 1);
+        const float *a0 = sA + buf * BK * C::LDS + ty * 4;
+        const float *b0 = sB + buf * BK * C::LDS + tx * C::CW;
+        // Fragments of the next k are read while this k's FMAs issue.
+        ulonglong2 a[2][C::TM / 4];
+        float b[2][C::TN];
+        auto load = [&](int k, int u) {
+#pragma unroll
+            for (int g = 0; g < C::TM / 4; ++g) a[u][g] = *(const ulonglong2 *)(a0 + k * C::LDS + g * 32);
+#pragma unroll
+            for (int h = 0; h < C::TN / C::CW; ++h) {
+                if constexpr (C::CW == 4) {
+                    const float4 v = *(const float4 *)(b0 + k * C::LDS + h * 64);
+                    b[u][4 * h] = v.x;
+                    b[u][4 * h + 1] = v.y;
+                    b[u][4 * h + 2] = v.z;
+                    b[u][4 * h + 3] = v.w;
+                } else {
+                    const float2 v = *(const float2 *)(b0 + k * C::LDS);
+                    b[u][0] = v.x;
+                    b[u][1] = v.y;
+                }
+            }
+        };
+        load(0, 0);
 #pragma unroll
         for (int k = 0; k < BK; ++k) {
-            const float4 a0 = *(const float4 *)&sm.A[buf][k][ty * 4];
-            const float4 a1 = *(const float4 *)&sm.A[buf][k][64 + ty * 4];
-            const float4 b0 = *(const float4 *)&sm.B[buf][k][tx * 4];
-            const float4 b1 = *(const float4 *)&sm.B[buf][k][64 + tx * 4];
-            const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-            const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+            if (k + 1 < BK) load(k + 1, (k + 1) & 1);
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
+            for (int j = 0; j < C::TN; ++j) {
+                const unsigned long long bj = pack2(b[k & 1][j], b[k & 1][j]);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+                for (int g = 0; g < C::TM / 4; ++g) {
+                    ffma2(acc[2 * g][j], a[k & 1][g].x, bj);
+                    ffma2(acc[2 * g + 1][j], a[k & 1][g].y, bj);
+                }
+            }
         }
         if (kt + 1 < nk) stash(buf ^ 1, kt + 1);
         __syncthreads();
@@ -88,55 +156,95 @@ __device__ __forceinline__ void simt_tile_mma(const float *__restrict__ X, int n
 // (a^2, 2a(1 - a), (1 - a)^2), or 2T - T^2 with T = aX, (-a^2, 2a, 0).  With
 // X^2 = acc + X - I/4 (acc = Y^2 of the centred operands) this is
 // k2 acc + (k2 + k1) X + (k0 - k2/4) I.
-__device__ __forceinline__ void simt_tile_epilogue(const float *__restrict__ Xold, float *__restrict__ Xnew, int np,
-                                                   int n, int r0, int c0, int flip, float alpha,
-                                                   const float acc[8][8], FF &ft, FF &fq) {
+template <int T>
+__device__ __forceinline__ void simt_tile_epilogue(const float *Xold, float *Xnew, int np, int n, int r0, int c0,
+                                                   int flip, float alpha,
+                                                   const unsigned long long (&acc)[SimtCfg<T>::TM / 2][SimtCfg<T>::TN],
+                                                   FF &ft, FF &fq) {
+    using C = SimtCfg<T>;
     const int tid = threadIdx.x;
     const float k2 = flip ? -alpha * alpha : alpha * alpha;
     const float kx = alpha * (2.0f - alpha);
     const float kd = flip ? 0.25f * alpha * alpha : (1.0f - alpha) * (1.0f - alpha) - 0.25f * alpha * alpha;
     const int tx = tid & 15, ty = tid >> 4;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int r = r0 + (i < 4 ? ty * 4 + i : 64 + ty * 4 + (i - 4));
+    for (int g = 0; g < C::TM / 4; ++g) {
+        const int rb = r0 + g * 32 + ty * 4;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int cb = c0 + (h == 0 ? tx * 4 : 64 + tx * 4);
-            float v[4];
-            const float4 xo = *(const float4 *)(Xold + (size_t)r * np + cb);
-            const float xov[4] = {xo.x, xo.y, xo.z, xo.w};
+        for (int h = 0; h < C::TN / C::CW; ++h) {
+            const int cb = c0 + h * 64 + tx * C::CW;
+            float v[4][C::CW];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const float s = acc[i][h * 4 + q];
-                const bool dg = (r == cb + q) && (r < n);
-                v[q] = fmaf(k2, s, fmaf(kx, xov[q], dg ? kd : 0.0f));
-            }
-            const bool all_owned = (r <= cb);
-            if (all_owned) {
-                *(float4 *)(Xnew + (size_t)r * np + cb) = make_float4(v[0], v[1], v[2], v[3]);
-            }
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int c = cb + q;
-                if (r > c) continue;
-                if (!all_owned) Xnew[(size_t)r * np + c] = v[q];
-                if (r < c) {
-                    Xnew[(size_t)c * np + r] = v[q];
-                    ff_add_sq(fq, v[q], 2.0f);
+            for (int i = 0; i < 4; ++i) {
+                const int r = rb + i;
+                float xo[C::CW];
+                if constexpr (C::CW == 4) {
+                    const float4 x = *(const float4 *)(Xold + (size_t)r * np + cb);
+                    xo[0] = x.x;
+                    xo[1] = x.y;
+                    xo[2] = x.z;
+                    xo[3] = x.w;
                 } else {
-                    ff_add(ft, v[q]);
-                    ff_add_sq(fq, v[q], 1.0f);
+                    const float2 x = *(const float2 *)(Xold + (size_t)r * np + cb);
+                    xo[0] = x.x;
+                    xo[1] = x.y;
                 }
+#pragma unroll
+                for (int q = 0; q < C::CW; ++q) {
+                    const float2 s2 = unpack2(acc[2 * g + (i >> 1)][h * C::CW + q]);
+                    const bool dg = (r == cb + q) && (r < n);
+                    v[i][q] = fmaf(k2, (i & 1) ? s2.y : s2.x, fmaf(kx, xo[q], dg ? kd : 0.0f));
+                }
+            }
+            if (rb + 3 < cb) {   // strictly above the diagonal: vector stores, direct and mirrored
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    float *p = Xnew + (size_t)(rb + i) * np + cb;
+                    if constexpr (C::CW == 4) *(float4 *)p = make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
+                    else *(float2 *)p = make_float2(v[i][0], v[i][1]);
+                }
+#pragma unroll
+                for (int q = 0; q < C::CW; ++q) {
+                    *(float4 *)(Xnew + (size_t)(cb + q) * np + rb) = make_float4(v[0][q], v[1][q], v[2][q], v[3][q]);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) ff_add_sq(fq, v[i][q], 2.0f);
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int q = 0; q < C::CW; ++q) {
+                        const int r = rb + i, c = cb + q;
+                        if (r > c) continue;
+                        Xnew[(size_t)r * np + c] = v[i][q];
+                        if (r < c) {
+                            Xnew[(size_t)c * np + r] = v[i][q];
+                            ff_add_sq(fq, v[i][q], 2.0f);
+                        } else {
+                            ff_add(ft, v[i][q]);
+                            ff_add_sq(fq, v[i][q], 1.0f);
+                        }
+                    }
             }
         }
     }
 }
 
-// Two CTAs per SM at 128 registers per thread (the comparator's throughput halves
-// at one; a launch bound forcing it makes the kernel spill and costs 4 %).
-__global__ void __launch_bounds__(SIMT_THREADS) k_simt_persistent(const __grid_constant__ RunParams p) {
+template <int T>
+__device__ __forceinline__ void simt_tile(const InstDesc &d, int n, int bi, int bj, int flip, float alpha,
+                                          float *stage, FF &ft, FF &fq) {
+    const float *X = d.xf[n & 1];
+    unsigned long long acc[SimtCfg<T>::TM / 2][SimtCfg<T>::TN];
+    simt_tile_mma<T>(X, d.np, d.n, bi * T, bj * T, stage, acc);
+    simt_tile_epilogue<T>(X, d.xf[(n + 1) & 1], d.np, d.n, bi * T, bj * T, flip, alpha, acc, ft, fq);
+}
+
+template <int TMAX>
+__global__ void __launch_bounds__(SIMT_THREADS, TMAX == 128 ? 2 : 4) k_simt_persistent(const __grid_constant__ RunParams p) {
     __shared__ RoundCtl rc;
-    __shared__ __align__(16) SimtSmem sm;
+    __shared__ __align__(16) SimtSmem<TMAX> sm;
+    static_assert(sizeof(sm.stage) >= (4 * MAX_BATCH + 4 * (SIMT_THREADS / 32)) * sizeof(double),
+                  "round sums reuse the staging buffers");
     if (threadIdx.x == 0) round_ctl_init(rc, p);
     __syncthreads();
     unsigned int target = 0;
@@ -154,7 +262,7 @@ __global__ void __launch_bounds__(SIMT_THREADS) k_simt_persistent(const __grid_c
         }
         first = false;
         // The operand staging buffers are idle here: use them for the sums.
-        double *sums = (double *)&sm.A[0][0][0];
+        double *sums = (double *)sm.stage;
         reduce_round_partials_block(rc, p, sums, sums + 4 * MAX_BATCH);
         if (threadIdx.x == 0) decide_round(rc, p, sums);
         __syncthreads();
@@ -164,14 +272,12 @@ __global__ void __launch_bounds__(SIMT_THREADS) k_simt_persistent(const __grid_c
             map_tile(rc, p.B, p.inst, g, i, job, tile);
             const InstDesc &d = p.inst[i];
             const int2 bt = p.tiles[d.tile_off + tile];
-            const int n = rc.layer[i];
-            const float *X = d.xf[n & 1];
-            float *Xn = d.xf[(n + 1) & 1];
-            float acc[8][8];
-            simt_tile_mma(X, d.np, d.n, bt.x * SIMT_T, bt.y * SIMT_T, sm, acc);
+            const int n = rc.layer[i], flip = rc.choice[i] == SP2_CHOICE_FLIP;
+            const float alpha = rc.alpha[i];
             FF ft = {0.f, 0.f}, fq = {0.f, 0.f};
-            simt_tile_epilogue(X, Xn, d.np, d.n, bt.x * SIMT_T, bt.y * SIMT_T, rc.choice[i] == SP2_CHOICE_FLIP,
-                               rc.alpha[i], acc, ft, fq);
+            if (TMAX >= 128 && d.simt_t == 128) simt_tile<TMAX >= 128 ? 128 : 32>(d, n, bt.x, bt.y, flip, alpha, sm.stage, ft, fq);
+            else if (TMAX >= 64 && d.simt_t == 64) simt_tile<TMAX >= 64 ? 64 : 32>(d, n, bt.x, bt.y, flip, alpha, sm.stage, ft, fq);
+            else simt_tile<32>(d, n, bt.x, bt.y, flip, alpha, sm.stage, ft, fq);
             // Deterministic block reduction of the tile partials.
             double t = ff_value(ft), q = ff_value(fq);
             for (int o = 16; o > 0; o >>= 1) {
@@ -197,15 +303,20 @@ __global__ void __launch_bounds__(SIMT_THREADS) k_simt_persistent(const __grid_c
     }
 }
 
+const void *simt_kernel(int tmax) {
+    return tmax == 128 ? (const void *)k_simt_persistent<128>
+                       : tmax == 64 ? (const void *)k_simt_persistent<64> : (const void *)k_simt_persistent<32>;
+}
+
 }  // namespace
 
-int simt_blocks_per_sm() {
+int simt_blocks_per_sm(int tmax) {
     int b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_simt_persistent, SIMT_THREADS, 0) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, simt_kernel(tmax), SIMT_THREADS, 0) != cudaSuccess) return 0;
     return b;
 }
 
-cudaError_t launch_simt_persistent(const RunParams &p, int grid, cudaStream_t s) {
+cudaError_t launch_simt_persistent(const RunParams &p, int tmax, int grid, cudaStream_t s) {
     void *args[] = {(void *)&p};
     // Cooperative launch in the attribute form (also capturable in a CUDA graph).
     cudaLaunchConfig_t cfg = {};
@@ -218,7 +329,7 @@ cudaError_t launch_simt_persistent(const RunParams &p, int grid, cudaStream_t s)
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelExC(&cfg, (const void *)k_simt_persistent, args);
+    return cudaLaunchKernelExC(&cfg, simt_kernel(tmax), args);
 }
 
 }  // namespace sp2i

@@ -43,8 +43,7 @@ constexpr int MAPS_PER_SLOT = 5;    // per operand slot: loads hi, hi, lo (64 x 
 constexpr int EPI_BOX_COLS = 16;    // store box: one epilogue warp's chunk of 32 rows x 16 columns
 constexpr int EPI_BOX_ROWS = 32;
 constexpr int TC_THREADS = 320;     // warp 0 TMA, warp 1 MMA, warps 2..9 epilogue (two per SM sub-partition)
-constexpr int SIMT_T = 128;         // FP32 SIMT tile (square)
-constexpr int SIMT_THREADS = 256;
+constexpr int SIMT_THREADS = 128;   // FP32 CUDA-core kernel: 8 x 16 threads on a square tile
 constexpr int MAX_BATCH = 128;
 constexpr int MAX_L = SP2_MAX_LAYERS_LIMIT;
 constexpr int INIT_BLOCKS_MAX = 1024;
@@ -107,6 +106,7 @@ struct InstDesc {
     uint16_t *yop;                    // slot s in {0,1}: hi, lo as for xop
     Part *part[3];                    // by layer n mod 3 (three deep for the dataflow schedule)
     int part_cap, fin_blocks;
+    int simt_t, pad_simt;             // FP32 path: tile side (simt_tile_side)
     const CUtensorMap *xmap;          // [nslots_x * MAPS_PER_SLOT]: per slot the K segments' loads op0, op1,
                                       // op2 = hi, hi, lo, then the epilogue's stores of hi and lo
     const CUtensorMap *ymap;          // [2 * MAPS_PER_SLOT]
@@ -148,12 +148,23 @@ cudaError_t launch_init_y(InstDesc *inst, int mode, int precision, cudaStream_t 
 int finalize_blocks();
 cudaError_t launch_finalize(InstDesc *inst, int B, int fin_blocks, int mode, cudaStream_t s);
 cudaError_t launch_fill_trivial(float *D, int n, float diag_value, cudaStream_t s);
-cudaError_t launch_simt_persistent(const RunParams &p, int grid, cudaStream_t s);
+// FP32 path: `tmax` is the largest tile side of the launch's instances.
+cudaError_t launch_simt_persistent(const RunParams &p, int tmax, int grid, cudaStream_t s);
 cudaError_t launch_tc_persistent(const RunParams &p, int cta_group, int grid, cudaStream_t s);
-int simt_blocks_per_sm();
+int simt_blocks_per_sm(int tmax);
 int tc_grid_size(int cta_group, int sm_count);
 size_t tc_smem_bytes();
 
 inline int round_up(int a, int b) { return (a + b - 1) / b * b; }
+
+// Side of the FP32 path's square tiles for an np x np instance.  Every element is the
+// same chain of FMAs whatever the side, so it is chosen for speed alone: small tiles
+// spread a small matrix over the SMs, large ones reuse a staged value more often (the
+// inner loop is bound by shared-memory reads below 128).  Microseconds per layer with
+// sides 32 / 64 / 128 (before: 128 only, scalar FMAs):
+//   np 256:  16 /  22 /  49 ( 43)    np 768:   38 /  44 /  95 ( 98)
+//   np 1024: 89 /  54 / 119 (122)    np 1280: 198 / 102 / 144 (150)
+//   np 1664: 375 / 187 / 180 (187)   np 3072: 1776 / 871 / 525 (651)
+inline int simt_tile_side(int np) { return np <= 768 ? 32 : np <= 1536 ? 64 : 128; }
 
 }  // namespace sp2i
