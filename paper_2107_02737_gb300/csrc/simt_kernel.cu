@@ -33,9 +33,12 @@ struct SimtCfg {
     static constexpr int FLOATS = 2 * 2 * BK * LDS;     // A and B, double-buffered
 };
 
+constexpr int max_floats(int a, int b) { return a > b ? a : b; }
+
+// A launch whose largest side is TMAX also runs tiles of the smaller sides.
 template <int TMAX>
 struct SimtSmem {
-    float stage[SimtCfg<TMAX>::FLOATS];
+    float stage[max_floats(SimtCfg<32>::FLOATS, max_floats(SimtCfg<TMAX >= 64 ? 64 : 32>::FLOATS, SimtCfg<TMAX>::FLOATS))];
     double red[SIMT_THREADS / 32][2];
 };
 
@@ -243,6 +246,10 @@ template <int TMAX>
 __global__ void __launch_bounds__(SIMT_THREADS, TMAX == 128 ? 2 : 4) k_simt_persistent(const __grid_constant__ RunParams p) {
     __shared__ RoundCtl rc;
     __shared__ __align__(16) SimtSmem<TMAX> sm;
+    static_assert(sizeof(sm.stage) >= sizeof(float) * SimtCfg<TMAX>::FLOATS &&
+                      (TMAX < 64 || sizeof(sm.stage) >= sizeof(float) * SimtCfg<64>::FLOATS) &&
+                      sizeof(sm.stage) >= sizeof(float) * SimtCfg<32>::FLOATS,
+                  "staging of every side the launch runs");
     static_assert(sizeof(sm.stage) >= (4 * MAX_BATCH + 4 * (SIMT_THREADS / 32)) * sizeof(double),
                   "round sums reuse the staging buffers");
     if (threadIdx.x == 0) round_ctl_init(rc, p);
