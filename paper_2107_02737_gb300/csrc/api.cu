@@ -41,13 +41,13 @@ EncodeTiledFn get_encode_fn() {
     return fn;
 }
 
-// 2-D map over an np x np 16-bit matrix, box 64 (K, inner) x 128 rows, 128B swizzle.
-bool encode_op_map(CUtensorMap *m, const void *base, int np, int precision) {
+// 2-D map over an np x np 16-bit matrix, box 64 (K, inner) x `rows` rows, 128B swizzle.
+bool encode_op_map(CUtensorMap *m, const void *base, int np, int precision, int rows) {
     EncodeTiledFn fn = get_encode_fn();
     if (!fn) return false;
     cuuint64_t dims[2] = {(cuuint64_t)np, (cuuint64_t)np};
     cuuint64_t strides[1] = {(cuuint64_t)np * 2};
-    cuuint32_t box[2] = {(cuuint32_t)TC_BK, (cuuint32_t)(TC_BN / 2)};
+    cuuint32_t box[2] = {(cuuint32_t)TC_BK, (cuuint32_t)rows};
     cuuint32_t estr[2] = {1, 1};
     CUresult r = fn(m, precision == SP2_BF16_SPLIT ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2,
                     const_cast<void *>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -71,10 +71,10 @@ bool encode_store_map(CUtensorMap *m, const void *base, int np) {
 }
 
 // The MAPS_PER_SLOT maps of one operand slot (matrices hi at `hi`, lo at hi + np^2).
-bool encode_slot_maps(CUtensorMap *m, const uint16_t *hi, int np, int precision) {
+bool encode_slot_maps(CUtensorMap *m, const uint16_t *hi, int np, int precision, int rows) {
     const size_t mat = (size_t)np * np;
     for (int k = 0; k < 3; ++k)
-        if (!encode_op_map(&m[k], hi + (k == 2 ? mat : 0), np, precision)) return false;
+        if (!encode_op_map(&m[k], hi + (k == 2 ? mat : 0), np, precision, rows)) return false;
     return encode_store_map(&m[3], hi, np) && encode_store_map(&m[4], hi + mat, np);
 }
 
@@ -154,16 +154,16 @@ struct Carver {
     }
 };
 
-// Tile tables: SIMT uses square 128-tiles with bi <= bj; the tensor-core path
-// uses 128 x 256 tiles containing at least one element with row <= column.
+// Tile tables: SIMT uses square tiles with bi <= bj; the tensor-core path uses
+// 128 cg x bn tiles containing at least one element with row <= column.
 // CTA b takes tiles b, b + grid, ..., so each run of `grid` consecutive tiles is
 // in flight together.  Tiles are ordered by 2048 x 2048 super-blocks (column
 // super-block, then row super-block, then column, then row) so that such a run
 // reads a compact set of row and column panels and the operand matrices, which
 // are larger than L2, are fetched from HBM about once per run.
-void build_tiles_uncached(int path, int np, int cg, std::vector<int2> &t) {
+void build_tiles_uncached(int path, int np, int cg, int tbn, std::vector<int2> &t) {
     const int bm = (path == PATH_SIMT) ? simt_tile_side(np) : TC_BM * cg;
-    const int bn = (path == PATH_SIMT) ? simt_tile_side(np) : TC_BN;
+    const int bn = (path == PATH_SIMT) ? simt_tile_side(np) : tbn;
     const int nbi = (np + bm - 1) / bm, nbj = (np + bn - 1) / bn;  // a last pair tile may overhang np
     const int sbi = 2048 / bm, sbj = 2048 / bn;  // tiles per super-block side
     std::vector<std::pair<long long, int2>> keyed;
@@ -178,33 +178,30 @@ void build_tiles_uncached(int path, int np, int cg, std::vector<int2> &t) {
     for (auto &k : keyed) t.push_back(k.second);
 }
 
-// The table for (path, np, cg) is built once per process (calls repeat the same sizes).
-void build_tiles(int path, int np, int cg, std::vector<int2> &t) {
+// The table for (path, np, cg, bn) is built once per process (calls repeat the same sizes).
+void build_tiles(int path, int np, int cg, int tbn, std::vector<int2> &t) {
     static std::mutex mu;
     static std::map<long long, std::vector<int2>> cache;
-    const long long key = ((long long)path * 4 + cg) * (1LL << 32) + np;
+    const long long key = (((long long)path * 4 + cg) * 512 + tbn) * (1LL << 32) + np;
     std::lock_guard<std::mutex> lock(mu);
     auto it = cache.find(key);
     if (it == cache.end()) {
         std::vector<int2> v;
-        build_tiles_uncached(path, np, cg, v);
+        build_tiles_uncached(path, np, cg, tbn, v);
         it = cache.emplace(key, std::move(v)).first;
     }
     t.insert(t.end(), it->second.begin(), it->second.end());
 }
 
 // Number of tiles of the table above, counted without building it.
-int ntiles_for(int path, int np, int cg) {
+int ntiles_for(int path, int np, int cg, int tbn) {
     const int bm = (path == PATH_SIMT) ? simt_tile_side(np) : TC_BM * cg;
-    const int bn = (path == PATH_SIMT) ? simt_tile_side(np) : TC_BN;
+    const int bn = (path == PATH_SIMT) ? simt_tile_side(np) : tbn;
     const int nbi = (np + bm - 1) / bm, nbj = (np + bn - 1) / bn;
     int count = 0;
     for (int bj = 0; bj < nbj; ++bj) count += std::min(nbi, ((bj + 1) * bn + bm - 1) / bm);
     return count;
 }
-
-// Partial records per layer: one per tile, per CTA of the tile.
-int parts_for(int path, int np, int cg) { return ntiles_for(path, np, cg) * (path == PATH_TC ? cg : 1); }
 
 // Must equal the device-side init_blocks_for: one partial per input-layer block.
 int init_blocks_host(int np) { return np < INIT_BLOCKS_MAX ? np : INIT_BLOCKS_MAX; }
@@ -212,7 +209,10 @@ int init_blocks_host(int np) { return np < INIT_BLOCKS_MAX ? np : INIT_BLOCKS_MA
 struct Plan {
     int mode, path, precision;
     bool dataflow = false;            // see flow_eligible
-    int cg = 1;                       // CTAs per tensor-core tile
+    int cg = 1, bn = TC_BN;           // tensor-core tile: CTAs and columns
+    int kwave = 1;                    // InstDesc::kwave
+    bool narrow = false;              // tiles narrower than the partial records' (see Part)
+    bool flow_blocks = false;         // dataflow: waits per block of X, not per layer
     int simt_tmax = 128;              // FP32 path: largest tile side of the instances
     std::vector<InstSpec> inst;       // non-trivial instances, in launch order
     std::vector<int> slots;           // nslots_x per instance
@@ -273,6 +273,13 @@ void adjoint_layout(int lmax, int stride, int &slots, int &s_out, int &k_out) {
     slots = k_out + s - 1;
 }
 
+// Partial records per layer: one per tile, per CTA of the tile; with narrow tiles those
+// of the 256 x 256 pair tiles.
+int parts_for(const Plan &pl, int np) {
+    const int cg = pl.narrow ? 2 : pl.cg, bn = pl.narrow ? TC_BN : pl.bn;
+    return ntiles_for(pl.path, np, cg, bn) * (pl.path == PATH_TC ? cg : 1);
+}
+
 size_t plan_bytes(const Plan &pl, std::vector<size_t> *offsets_unused = nullptr) {
     (void)offsets_unused;
     Carver c(nullptr);
@@ -283,14 +290,17 @@ size_t plan_bytes(const Plan &pl, std::vector<size_t> *offsets_unused = nullptr)
     c.take(sizeof(InstCtl) * B);          // their initial state, copied in before every replay
     c.take(sizeof(InstDesc) * B);
     int tiles = 0;
-    for (auto &s : pl.inst) tiles += ntiles_for(pl.path, round_up(s.n, PAD), pl.cg);
+    for (auto &s : pl.inst) {
+        tiles += ntiles_for(pl.path, round_up(s.n, PAD), pl.cg, pl.bn);
+        if (pl.narrow) tiles += ntiles_for(pl.path, round_up(s.n, PAD), 2, TC_BN);
+    }
     c.take(sizeof(int2) * tiles);
     c.take(sizeof(int) * (MAX_L + 1));    // forced choices
     c.take(sizeof(double) * (MAX_L + 1)); // forced expansions
     for (int i = 0; i < B; ++i) {
         const int np = round_up(pl.inst[i].n, PAD);
         if (pl.dataflow) {
-            c.take(sizeof(unsigned int) * ntiles_for(pl.path, np, pl.cg));      // tile completions
+            c.take(sizeof(unsigned int) * ntiles_for(pl.path, np, pl.cg, pl.bn));      // tile completions
             c.take(sizeof(int) * 2 * (size_t)flow_nblk(np) * flow_nblk(np));  // block sources
         }
         if (pl.path == PATH_TC) {
@@ -302,10 +312,12 @@ size_t plan_bytes(const Plan &pl, std::vector<size_t> *offsets_unused = nullptr)
     for (int i = 0; i < B; ++i) {
         const int np = round_up(pl.inst[i].n, PAD);
         const size_t mat = (size_t)np * np;
-        const int cap = std::max(parts_for(pl.path, np, pl.cg), initb);
-        c.take(sizeof(Part) * cap);
-        c.take(sizeof(Part) * cap);
-        c.take(sizeof(Part) * cap);
+        const int cap = std::max(parts_for(pl, np), initb);
+        for (int k = 0; k < 3; ++k) c.take(sizeof(Part) * cap);
+        if (pl.path == PATH_TC) {
+            c.take(sizeof(float) * np);
+            c.take(sizeof(float) * np);
+        }
         c.take(sizeof(double2) * FIN_BLOCKS_MAX);
         c.take(mat * 4);
         c.take(mat * 4);
@@ -397,6 +409,7 @@ struct Prepared {
     unsigned int *d_tile_done = nullptr;   // dataflow: per-tile completion counters
     int *d_blk_src = nullptr;              // dataflow: block sources
     int flow_tiles = 0, flow_nb = 0;
+    int units = 0;                   // RunParams::units
     int fin_blocks = 0;              // output kernel blocks per instance
     InstCtl *d_ctl = nullptr;        // B live control blocks
     InstCtl *d_ctl_init = nullptr;   // B initial control blocks
@@ -414,7 +427,7 @@ struct Prepared {
 struct LaunchGeometry {
     bool known = false;
     DeviceInfo di;
-    int grid_cg[3] = {0, 0, 0};
+    int grid_tc[3][3] = {};         // CTAs of a resident grid: [CTAs per tile][64, 128, 256 columns]
     int simt_per_sm[3] = {0, 0, 0};   // resident CTAs per SM with tiles up to 32, 64, 128
 };
 bool launch_geometry(LaunchGeometry &g) {
@@ -432,14 +445,50 @@ bool launch_geometry(LaunchGeometry &g) {
         e.di = query_device();
         if (e.di.err != cudaSuccess) return false;
         if (e.di.major == 10 && e.di.minor == 3) {
-            e.grid_cg[2] = tc_grid_size(2, e.di.sm);
-            e.grid_cg[1] = tc_grid_size(1, e.di.sm);
+            e.grid_tc[1][0] = tc_grid_size(1, 64, e.di.sm);
+            e.grid_tc[2][1] = tc_grid_size(2, 128, e.di.sm);
+            for (int cg = 1; cg <= 2; ++cg) e.grid_tc[cg][2] = tc_grid_size(cg, 256, e.di.sm);
             for (int k = 0; k < 3; ++k) e.simt_per_sm[k] = simt_blocks_per_sm(32 << k);
         }
         e.known = true;
     }
     g = e;
     return true;
+}
+
+// Tiles of one round of the plan (a response computes two per position).
+int round_tiles(const Plan &pl, int cg, int bn) {
+    int t = 0;
+    for (auto &sp : pl.inst) t += ntiles_for(PATH_TC, round_up(sp.n, PAD), cg, bn);
+    return pl.mode == MODE_RESPONSE ? 2 * t : t;
+}
+
+// A lone density solve takes narrower tiles where 256 x 256 pair tiles would leave SMs without work: the
+// narrowest whose tiles all run at once.  X is the same with every shape as long as
+// every tile walks K upward, which pair tiles do when an instance has no more of them
+// than the device runs at once.  A tile's K loop is bound by its operand copies (about
+// 50 bytes per cycle and SM), so 256 x 128 tiles, whose CTAs share B, beat 128 x 128.
+// Microseconds per layer, 128 x 64 / 256 x 64 / 128 x 128 / 256 x 128 / 256 x 256
+// (before: 256 x 256 only):
+//   N 100:  12.5 / 12.5 / 14.8 / 15.1 / 21.6 (24.6)
+//   N 600:  17.5 / 17.6 / 20.7 / 20.0 / 27.6 (35.0)
+//   N 1280: 24.7 / 26.3 / 27.9 / 28.2 / 36.0 (44.7)
+//   N 1537: 50.4 /  --  / 34.2 / 30.6 / 41.1 (50.6)
+//   N 2048: 59.8 /  --  / 39.2 / 35.6 / 46.6 (56.9)
+//   N 2304: 92.1 /  --  / 69.8 /  --  / 49.3 (61.3)
+void narrow_tiles(Plan &pl, const LaunchGeometry &geo, int &grid) {
+    for (auto &sp : pl.inst)
+        if (ntiles_for(PATH_TC, round_up(sp.n, PAD), 2, TC_BN) > pl.kwave) return;
+    for (int cg = 1; cg <= 2; ++cg) {   // 128 x 64, then 256 x 128
+        const int bn = 64 * cg, g = geo.grid_tc[cg][cg - 1];
+        if (round_tiles(pl, cg, bn) > g / cg) continue;
+        pl.cg = cg;
+        pl.bn = bn;
+        pl.kwave = 1 << 30;
+        pl.narrow = true;
+        grid = g;
+        return;
+    }
 }
 
 sp2_status choose_launch(Plan &pl, int want, int &grid) {
@@ -451,22 +500,32 @@ sp2_status choose_launch(Plan &pl, int want, int &grid) {
     grid = 0;
     if (pl.path == PATH_TC) {
         if (want == 0 || want == 2) {
-            grid = geo.grid_cg[2];
+            grid = geo.grid_tc[2][2];
             pl.cg = 2;
+            pl.bn = TC_BN;
         }
         if (grid <= 0) {
             if (want == 2) return SP2_ERR_UNSUPPORTED;
-            grid = geo.grid_cg[1];
+            grid = geo.grid_tc[1][2];
             pl.cg = 1;
+            pl.bn = TC_BN;
         }
         if (grid <= 0) return SP2_ERR_UNSUPPORTED;
+        // A device constant, so that an instance's tiles walk K the same way in a
+        // batch as alone (the accumulation order, and so the bits, follow the tile).
+        pl.kwave = std::max(1, grid / pl.cg);
+        if (want == 0 && pl.cg == 2 && pl.dataflow) narrow_tiles(pl, geo, grid);
+        // No more CTAs than a layer has tiles: the rest would only poll.
+        const int tiles = round_tiles(pl, pl.cg, pl.bn);
+        pl.flow_blocks = pl.dataflow && pl.bn == TC_BN && tiles > grid / pl.cg;
+        if (tiles < grid / pl.cg) grid = std::max(1, tiles) * pl.cg;
     } else {
         pl.simt_tmax = simt_tile_side(pl.max_np);
         const int per_sm = geo.simt_per_sm[pl.simt_tmax == 32 ? 0 : pl.simt_tmax == 64 ? 1 : 2];
         if (per_sm <= 0) return SP2_ERR_UNSUPPORTED;
         // No more CTAs than a round has tiles: the grid barrier costs less.
         int tiles = 0;
-        for (auto &sp : pl.inst) tiles += ntiles_for(PATH_SIMT, round_up(sp.n, PAD), 1);
+        for (auto &sp : pl.inst) tiles += ntiles_for(PATH_SIMT, round_up(sp.n, PAD), 1, 0);
         grid = std::max(1, std::min(per_sm * di.sm, tiles));
     }
     return SP2_OK;
@@ -491,11 +550,15 @@ sp2_status prepare(Prepared &P, const sp2_opts &o, double tol, void *ws, size_t 
     InstCtl *d_ctl = (InstCtl *)c.take(sizeof(InstCtl) * B);
     InstCtl *d_ctl_init = (InstCtl *)c.take(sizeof(InstCtl) * B);
     InstDesc *d_inst = (InstDesc *)c.take(sizeof(InstDesc) * B);
-    std::vector<std::vector<int2>> tiles(B);
+    std::vector<std::vector<int2>> tiles(B), units(B);   // units: the partial records' pair tiles (narrow)
     int total_tiles = 0;
     for (int i = 0; i < B; ++i) {
-        build_tiles(pl.path, round_up(pl.inst[i].n, PAD), pl.cg, tiles[i]);
+        build_tiles(pl.path, round_up(pl.inst[i].n, PAD), pl.cg, pl.bn, tiles[i]);
         total_tiles += (int)tiles[i].size();
+        if (pl.narrow) {
+            build_tiles(pl.path, round_up(pl.inst[i].n, PAD), 2, TC_BN, units[i]);
+            total_tiles += (int)units[i].size();
+        }
     }
     int2 *d_tiles = (int2 *)c.take(sizeof(int2) * total_tiles);
     int *d_forced = (int *)c.take(sizeof(int) * (MAX_L + 1));
@@ -545,12 +608,13 @@ sp2_status prepare(Prepared &P, const sp2_opts &o, double tol, void *ws, size_t 
         d.n = n;
         d.np = np;
         d.ntiles = (int)tiles[i].size();
-        d.parts = d.ntiles * (pl.path == PATH_TC ? pl.cg : 1);
-        // A device constant, so that an instance's tiles walk K the same way in a
-        // batch as alone (the accumulation order, and so the bits, follow the tile).
-        d.kwave = (pl.path == PATH_TC) ? std::max(1, P.grid / pl.cg) : 1;
+        d.parts = parts_for(pl, np);
+        d.kwave = (pl.path == PATH_TC) ? pl.kwave : 1;
         d.tile_off = (int)h_tiles.size();
         h_tiles.insert(h_tiles.end(), tiles[i].begin(), tiles[i].end());
+        d.unit_off = (int)h_tiles.size();
+        h_tiles.insert(h_tiles.end(), units[i].begin(), units[i].end());
+        if (pl.narrow) P.units = d.parts;
         d.n_occ = sp.n_occ;
         d.nforced = -1;
         d.nslots_x = pl.slots[i];
@@ -558,10 +622,10 @@ sp2_status prepare(Prepared &P, const sp2_opts &o, double tol, void *ws, size_t 
         d.fin_blocks = P.fin_blocks;
         d.simt_t = (pl.path == PATH_SIMT) ? simt_tile_side(np) : 0;
         d.ctl = d_ctl + i;
-        d.part[0] = (Part *)c.take(sizeof(Part) * d.part_cap);
-        d.part[1] = (Part *)c.take(sizeof(Part) * d.part_cap);
-        d.part[2] = (Part *)c.take(sizeof(Part) * d.part_cap);
-        if (pl.dataflow) {
+        for (int k = 0; k < 3; ++k) d.part[k] = (Part *)c.take(sizeof(Part) * d.part_cap);
+        if (pl.path == PATH_TC)
+            for (int k = 0; k < 2; ++k) d.pdiag[k] = (float *)c.take(sizeof(float) * np);
+        if (pl.flow_blocks) {
             std::vector<int> src;
             build_block_sources(np, pl.cg, tiles[i], src);
             put(d_src[i], src.data(), sizeof(int) * src.size());
@@ -577,7 +641,7 @@ sp2_status prepare(Prepared &P, const sp2_opts &o, double tol, void *ws, size_t 
             // slot's two matrices (hi, lo), then the epilogue's store maps of hi and lo.
             for (int sl = 0; sl < d.nslots_x; ++sl)
                 if (!encode_slot_maps(&h_xmaps[i][(size_t)sl * MAPS_PER_SLOT], d.xop + (size_t)sl * 2 * mat, np,
-                                      pl.precision))
+                                      pl.precision, tc_box_rows(pl.cg, pl.bn)))
                     return SP2_ERR_UNSUPPORTED;
             if (pl.ckpt_s[i] > 0) {
                 d.ckpt_s = pl.ckpt_s[i];
@@ -594,7 +658,7 @@ sp2_status prepare(Prepared &P, const sp2_opts &o, double tol, void *ws, size_t 
                 h_ymaps[i].resize(2 * MAPS_PER_SLOT);
                 for (int sl = 0; sl < 2; ++sl)
                     if (!encode_slot_maps(&h_ymaps[i][(size_t)sl * MAPS_PER_SLOT], d.yop + (size_t)sl * 2 * mat, np,
-                                          pl.precision))
+                                          pl.precision, tc_box_rows(pl.cg, pl.bn)))
                         return SP2_ERR_UNSUPPORTED;
             }
         }
@@ -765,18 +829,21 @@ sp2_status enqueue(const Prepared &P, cudaStream_t s, cudaEvent_t *ev, bool fres
     rp.mode = pl.mode;
     rp.precision = pl.precision;
     rp.max_layers = P.o.max_layers;
+    rp.units = P.units;
+    rp.stat_done = (unsigned int *)(P.d_sync + 12);
     // Device hook: CTA 0 withholds its first barrier arrival (test_hook 1, or 3 in a CTA-pair launch).
     rp.test_hook = (P.o.test_hook == 1 || (P.o.test_hook == 3 && pl.path == PATH_TC && pl.cg == 2)) ? 1 : 0;
-    rp.publish = (pl.mode == MODE_DENSITY && pl.path == PATH_TC && !pl.dataflow) ? 1 : 0;
     if (pl.dataflow) {
-        rp.dataflow = 1;
+        rp.dataflow = RUN_FLOW;
         rp.nblk = P.flow_nb;
         rp.tile_done = P.d_tile_done;
         rp.layer_done = (unsigned int *)(P.d_sync + 8);
-        rp.blk_src = P.d_blk_src;
+        rp.blk_src = pl.flow_blocks ? P.d_blk_src : nullptr;
     }
+    // A density batch: its own dataflow schedule.
+    if (pl.mode == MODE_DENSITY && pl.path == PATH_TC && !pl.dataflow) rp.dataflow = RUN_BATCH;
     if (ev) CK(cudaEventRecord(ev[1], s));
-    CK(pl.path == PATH_TC ? launch_tc_persistent(rp, pl.cg, P.grid, s) : launch_simt_persistent(rp, pl.simt_tmax, P.grid, s));
+    CK(pl.path == PATH_TC ? launch_tc_persistent(rp, pl.cg, pl.bn, P.grid, s) : launch_simt_persistent(rp, pl.simt_tmax, P.grid, s));
     if (ev) CK(cudaEventRecord(ev[2], s));
     CK(launch_finalize(P.d_inst, B, P.fin_blocks, pl.mode == MODE_APPLY ? MODE_DENSITY : pl.mode, s));
     if (ev) CK(cudaEventRecord(ev[3], s));
@@ -1009,11 +1076,16 @@ size_t bytes_for(int mode, const std::vector<int> &ns, int layers, const sp2_opt
     }
     if (pl.inst.empty()) return 0;
     set_flow(pl);
-    pl.cg = 1;
-    const size_t b1 = plan_bytes(pl);
-    pl.cg = 2;
-    const size_t b2 = plan_bytes(pl);
-    return b1 > b2 ? b1 : b2;  // the tile shape is chosen per device at run time
+    // The tile shape is chosen per device at run time.
+    size_t most = 0;
+    for (int cg = 1; cg <= 2; ++cg)
+        for (int bn = 64; bn <= TC_BN; bn *= 2) {
+            pl.cg = cg;
+            pl.bn = bn;
+            pl.narrow = bn < TC_BN;
+            most = std::max(most, plan_bytes(pl));
+        }
+    return most;
 }
 
 // Tile shape chosen by timing, per (precision, sorted sizes); process-wide.

@@ -421,28 +421,6 @@ __global__ void __launch_bounds__(AUX_THREADS) k_init_x(InstDesc *inst, int user
     }
 }
 
-// The 16-bit split (hi, lo) of two adjacent values, as packed pairs (element j in
-// the low half): the same values as split2 gives one at a time, from conversions
-// of two floats at once and exact scaling in the 16-bit domain.
-template <int PREC, int SHIFT>
-__device__ __forceinline__ void split2_pair(float a, float b, uint32_t &hi, uint32_t &lo) {
-    if (PREC == SP2_FP16_SPLIT) {
-        const __half2 h = __floats2half2_rn(a, b);
-        const float2 hf = __half22float2(h);
-        const __half2 hs = __hmul2(h, __float2half2_rn((float)(1 << SHIFT)));   // exact (|x| <= 1)
-        const __half2 l = __floats2half2_rn(__fsub_rn(a, hf.x) * (float)(1 << SHIFT),
-                                            __fsub_rn(b, hf.y) * (float)(1 << SHIFT));
-        hi = *reinterpret_cast<const uint32_t *>(&hs);
-        lo = *reinterpret_cast<const uint32_t *>(&l);
-    } else {
-        const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-        const float2 hf = __bfloat1622float2(h);
-        const __nv_bfloat162 l = __floats2bfloat162_rn(__fsub_rn(a, hf.x), __fsub_rn(b, hf.y));
-        hi = *reinterpret_cast<const uint32_t *>(&h);
-        lo = *reinterpret_cast<const uint32_t *>(&l);
-    }
-}
-
 // X_0 on the tensor-core path, from the lower triangle of H.  A tile (ti, tj) below
 // the diagonal gives X_0 there, its FP32 master (the layers and the output read
 // the master on and below the diagonal only) and the split operands of

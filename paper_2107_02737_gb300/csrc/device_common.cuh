@@ -118,6 +118,28 @@ __device__ __forceinline__ void split2(float x, uint16_t &hi, uint16_t &lo) {
     if (PREC == SP2_FP16_SPLIT) split_fp16<SHIFT>(x, hi, lo);
     else split_bf16(x, hi, lo);
 }
+// The 16-bit split (hi, lo) of two adjacent values, as packed pairs (element j in
+// the low half): the same values as split2 gives one at a time, from conversions
+// of two floats at once and exact scaling in the 16-bit domain.
+template <int PREC, int SHIFT>
+__device__ __forceinline__ void split2_pair(float a, float b, uint32_t &hi, uint32_t &lo) {
+    if (PREC == SP2_FP16_SPLIT) {
+        const __half2 h = __floats2half2_rn(a, b);
+        const float2 hf = __half22float2(h);
+        const __half2 hs = __hmul2(h, __float2half2_rn((float)(1 << SHIFT)));   // exact (|x| <= 1)
+        const __half2 l = __floats2half2_rn(__fsub_rn(a, hf.x) * (float)(1 << SHIFT),
+                                            __fsub_rn(b, hf.y) * (float)(1 << SHIFT));
+        hi = *reinterpret_cast<const uint32_t *>(&hs);
+        lo = *reinterpret_cast<const uint32_t *>(&l);
+    } else {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+        const float2 hf = __bfloat1622float2(h);
+        const __nv_bfloat162 l = __floats2bfloat162_rn(__fsub_rn(a, hf.x), __fsub_rn(b, hf.y));
+        hi = *reinterpret_cast<const uint32_t *>(&h);
+        lo = *reinterpret_cast<const uint32_t *>(&l);
+    }
+}
+
 // Factor that turns an accumulated product back into X X (resp = 0) or X Y (resp = 1).
 template <int PREC>
 __host__ __device__ __forceinline__ float product_unscale(bool resp) {
@@ -190,6 +212,7 @@ __device__ __forceinline__ float *xmaster(const InstDesc &d, int n, bool recompu
 // so no broadcast between CTAs is needed; CTA 0 alone writes the statistics.
 // ---------------------------------------------------------------------------
 struct RoundCtl {
+    const InstDesc *inst;            // the launch's instances (a lone one: a copy in shared memory)
     int abort;
     int total;                       // tiles in this round over all instances
     int phase;                       // adjoint: 0 forward, 1 reverse
@@ -206,20 +229,23 @@ struct RoundCtl {
     unsigned char ran[MAX_BATCH];    // instance computed a layer in the previous round
     double ehist[MAX_BATCH][2];
     double wprev[MAX_BATCH];         // ||Y_n||_F^2 of the operands of the current square
+    double inv_n[MAX_BATCH];         // 1 / n, rounded
     double coff[MAX_BATCH];          // c_n: true X_n = stored X_n + c_n I
     signed char chist[MAX_L + 2];    // adjoint (B = 1): choice that produced X_n
     double chist_c[MAX_L + 2];       // adjoint (B = 1): c_n per layer
     float chist_a[MAX_L + 2];        // adjoint (B = 1): a_n of the layer that produced X_n
     float alpha[MAX_BATCH];          // a of the layer computed this round (1 = plain)
     float xl[MAX_BATCH], xh[MAX_BATCH];  // accelerated chain: images of eps_lumo, eps_homo
-    int flow_go;                     // dataflow schedule: the previous layer is complete
+    int flow_go[2];                  // dataflow schedule, by layer parity: 1 run the layer, 0 stop
+    unsigned char degenerate[MAX_BATCH];   // no spread of the spectrum (set by the input layer)
 };
 
 __host__ __device__ __forceinline__ int layer_rule(double t, double q, double n_occ) {
     return fabs(q - n_occ) <= fabs(2.0 * t - q - n_occ) ? SP2_CHOICE_SQUARE : SP2_CHOICE_FLIP;
 }
 
-__device__ __forceinline__ void round_ctl_init(RoundCtl &rc, const RunParams &p) {
+__device__ __forceinline__ void round_ctl_init(RoundCtl &rc, const RunParams &p, const InstDesc *inst) {
+    rc.inst = inst;
     rc.abort = 0;
     rc.total = 0;
     rc.phase = 0;
@@ -234,10 +260,12 @@ __device__ __forceinline__ void round_ctl_init(RoundCtl &rc, const RunParams &p)
         rc.jobs[i] = 0;
         rc.choice[i] = SP2_CHOICE_INPUT;
         rc.active[i] = (ctl->status == 0) ? 1 : 0;
+        rc.degenerate[i] = ctl->degenerate ? 1 : 0;
         rc.ran[i] = 0;
         rc.ehist[i][0] = rc.ehist[i][1] = 0.0;
         rc.wprev[i] = 0.0;
         rc.coff[i] = 0.0;
+        rc.inv_n[i] = 1.0 / (double)p.inst[i].n;
         rc.alpha[i] = 1.0f;
         // Images of the estimated interval under the input layer, clipped to
         // [0, 1]; (0, 1) keeps every a_n = 1, the plain chain.
@@ -258,67 +286,48 @@ __device__ __forceinline__ void round_ctl_init(RoundCtl &rc, const RunParams &p)
     rc.chist_a[0] = 1.0f;
 }
 
-// One warp: the sums of instance i's partial records of layer n, lane l adding
-// entries l, l + 32, ... in increasing order, then a fixed shuffle tree (valid in
-// lane 0).  The order depends only on the instance's own records, so every CTA --
-// and a batch or a lone call alike -- gets the same bits and takes the same decision.
-__device__ __forceinline__ void sum_layer_partials(const RunParams &p, int i, int n, int lane, double (&a)[4]) {
-    const InstDesc &d = p.inst[i];
+// One warp: the sum of value c (Tr X, ||X||_F^2, ||Y||_F^2, Tr P) over instance d's
+// partial records of layer n, lane l adding entries l, l + 32, ... in increasing order,
+// then a fixed shuffle tree (valid in lane 0).  The order depends only on the
+// instance's own records, so every CTA -- and a batch or a lone call alike -- gets the
+// same bits and takes the same decision.
+__device__ __forceinline__ double sum_layer_value(const InstDesc &d, int n, int c, int lane) {
     const int cnt = (n == 0) ? d.ctl->init_parts : d.parts;
-    const Part *part = d.part[n % 3];
-    a[0] = a[1] = a[2] = a[3] = 0.0;
+    const double *part = &d.part[n % 3]->t + c;
+    double a = 0.0;
 #pragma unroll 4
-    for (int k = lane; k < cnt; k += 32) {
-        const Part v = part[k];
-        a[0] += v.t;
-        a[1] += v.q;
-        a[2] += v.w;
-        a[3] += v.p;
-    }
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-        for (int o = 16; o > 0; o >>= 1) a[c] += __shfl_down_sync(0xffffffffu, a[c], o);
+    for (int k = lane; k < cnt; k += 32) a += __ldcg(part + 4 * (size_t)k);
+    // Steps that would only add the zeros of lanes without an entry are left out: an FP64
+    // addition takes some 400 cycles here.
+    int o = 16;
+    while (o >= cnt && o > 1) o >>= 1;
+#pragma unroll 1
+    for (; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+    return a;
 }
 
-// The sums of the layer instance i just finished.
-__device__ __forceinline__ void sum_instance_partials(const RoundCtl &rc, const RunParams &p, int i, int lane,
-                                                      double (&a)[4]) {
-    sum_layer_partials(p, i, rc.layer[i] + (rc.ran[i] ? 1 : 0), lane, a);
+// The four sums, by one warp.
+__device__ __forceinline__ void sum_layer_partials(const InstDesc &d, int n, int lane, double (&a)[4]) {
+#pragma unroll 1
+    for (int c = 0; c < 4; ++c) {
+        const double v = sum_layer_value(d, n, c, lane);
+        if (c == 0) a[0] = v;
+        else if (c == 1) a[1] = v;
+        else if (c == 2) a[2] = v;
+        else a[3] = v;
+    }
 }
 
 // All threads of a CTA: the sums, for every instance still running, of the
 // partials of the layer just finished into sums[4 i .. 4 i + 3] (shared memory),
-// one warp per instance (warp w takes instances w, w + nwarps, ...).  In a density
-// batch's round schedule the CTA that completed an instance's layer has already
-// published these sums (same function, same order, same bits): they are read back.
-// `sums` is followed by MAX_BATCH ints of scratch (the decision's buffer, free here).
+// one warp per instance (warp w takes instances w, w + nwarps, ...).
 __device__ inline void reduce_round_partials(const RoundCtl &rc, const RunParams &p, double *sums) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
     if (rc.phase == 1) return;
-    int *got = (int *)(sums + 4 * MAX_BATCH);
-    // Published sums first, one thread per instance, every load in flight at once.
-    for (int i = threadIdx.x; i < p.B; i += blockDim.x) {
-        int ok = 0;
-        const int n = rc.layer[i] + (rc.ran[i] ? 1 : 0);
-        if (p.publish && rc.active[i] && n > 0) {
-            const InstCtl *ctl = p.inst[i].ctl;
-            const int pn = __ldcg(&ctl->psum_n);
-            double v[4];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) v[c] = __ldcg(&ctl->psum[c]);
-            if (pn == n) {
-#pragma unroll
-                for (int c = 0; c < 4; ++c) sums[i * 4 + c] = v[c];
-                ok = 1;
-            }
-        }
-        got[i] = ok;
-    }
-    __syncthreads();
     for (int i = wid; i < p.B; i += nw) {
-        if (!rc.active[i] || got[i]) continue;
+        if (!rc.active[i]) continue;
         double a[4];
-        sum_layer_partials(p, i, rc.layer[i] + (rc.ran[i] ? 1 : 0), lane, a);
+        sum_layer_partials(rc.inst[i], rc.layer[i] + (rc.ran[i] ? 1 : 0), lane, a);
         if (lane == 0)
             for (int c = 0; c < 4; ++c) sums[i * 4 + c] = a[c];
     }
@@ -340,7 +349,7 @@ __device__ inline void decide_round(RoundCtl &rc, const RunParams &p, const doub
         return;
     }
     if (rc.phase == 1) {  // adjoint reverse sweep (B == 1); layer[0] counts reverse rounds done
-        const InstDesc &d0 = p.inst[0];
+        const InstDesc &d0 = rc.inst[0];
         if (rc.rec_mode) {
             rc.rec_top += 1;  // X_{rec_top + 1} was recomputed
         } else {
@@ -375,7 +384,7 @@ __device__ inline void decide_round(RoundCtl &rc, const RunParams &p, const doub
     int acc = 0;
     rc.prefix[0] = 0;
     for (int i = 0; i < p.B; ++i) {
-        const int width = decide_instance(rc, p, sums, i, writer);
+        const int width = decide_instance(rc, p, sums + 4 * i, i, writer);
         if (width < 0) return;
         acc += width;
         rc.prefix[i + 1] = acc;
@@ -386,13 +395,13 @@ __device__ inline void decide_round(RoundCtl &rc, const RunParams &p, const doub
 // Compiled out of line: inlined into the persistent kernels it raises their
 // register allocation (the FP32 kernel then drops from two CTAs per SM to one).
 static __device__ __noinline__ int decide_instance(RoundCtl &rc, const RunParams &p, const double *sums, int i, bool writer) {
-    const InstDesc &d = p.inst[i];
+    const InstDesc &d = rc.inst[i];
     InstCtl *ctl = d.ctl;
     int width = 0;
     if (rc.active[i]) {
         if (rc.ran[i]) rc.layer[i] += 1;
         const int n = rc.layer[i];
-        const double ts = sums[i * 4 + 0], qs = sums[i * 4 + 1], ws = sums[i * 4 + 2], ps = sums[i * 4 + 3];
+        const double ts = sums[0], qs = sums[1], ws = sums[2], ps = sums[3];   // instance i's
         const int made = (n == 0) ? SP2_CHOICE_INPUT : rc.choice[i];
         // Accumulator bias of the square that made X_n: in exact arithmetic
         // Tr(Y^2) = ||Y||_F^2 for the symmetric operand Y, so the deficit of the
@@ -404,7 +413,11 @@ static __device__ __noinline__ int decide_instance(RoundCtl &rc, const RunParams
         double c = 0.0;
         const float a_made = (n == 0) ? 1.0f : rc.alpha[i];
         if (n > 0) {
-            const double gam = (rc.wprev[i] - ps) / (double)d.n;
+            // (wprev - ps) / n, correctly rounded from the rounded reciprocal by one
+            // residual step (Markstein's theorem): three FP64 operations.
+            const double dev = rc.wprev[i] - ps, inv = rc.inv_n[i];
+            const double g0 = dev * inv;
+            const double gam = isfinite(g0) ? fma(fma(-g0, (double)d.n, dev), inv, g0) : g0;
             const double a2 = (double)a_made * (double)a_made;
             c = (made == SP2_CHOICE_SQUARE) ? a2 * gam : -a2 * gam;
         }
@@ -435,7 +448,7 @@ static __device__ __noinline__ int decide_instance(RoundCtl &rc, const RunParams
         if (!isfinite(t) || !isfinite(q)) {
             stop = true;
             status = SP2_ERR_NONFINITE;
-        } else if (ctl->degenerate) {
+        } else if (rc.degenerate[i]) {
             stop = true;
             status = SP2_ERR_NOT_CONVERGED;
             reason = SP2_STOP_MAX;
@@ -529,7 +542,7 @@ __device__ inline void decide_round_parallel(RoundCtl &rc, const RunParams &p, c
     __syncthreads();
     if (rc.abort) return;
     const bool writer = (blockIdx.x == 0);
-    for (int i = threadIdx.x; i < p.B; i += blockDim.x) wbuf[i] = decide_instance(rc, p, sums, i, writer);
+    for (int i = threadIdx.x; i < p.B; i += blockDim.x) wbuf[i] = decide_instance(rc, p, sums + 4 * i, i, writer);
     __syncthreads();
     if (threadIdx.x == 0) {
         int acc = 0;

@@ -46,16 +46,18 @@ constexpr int XS_RING = 8;
 constexpr uint32_t XS_A_BYTES = 128 * TC_BK * 2;   // 16 KB: this CTA's 128 rows of one K block
 constexpr uint32_t XS_B_BYTES = 64 * TC_BK * 2;    // 8 KB: this CTA's 64 of the tile's 128 columns
 constexpr uint32_t XS_STAGE_BYTES = XS_A_BYTES + XS_B_BYTES;
-constexpr int XS_MAX_ST = 4;
 
 // Schedule of one tile, fixed at compile time by the slice count S (so that the
-// single MMA thread issues from registers, without table look-ups).  Sub-pass 0
-// holds stages (A_s, B_s), s < min(S, 4), and issues every product of levels
-// 0..3 into accumulator l = s + t.  With S >= 5 two more sub-passes (phase B)
-// issue the products of levels 4 and 5 into accumulators 2 and 3:
-//   sub-pass 1: stages (A2, B0), (A3, B1), (A4, B2) [, (A5, -)]
-//   sub-pass 2: stages (A0, B3), (A1, B4) [, (A2, B5)]
-// so that no K block needs more than four 24 KB stages.
+// MMA warp issues without table look-ups).  Sub-pass 0 holds stages (A_s, B_s),
+// s < min(S, 4), and issues every product of levels 0..3 into accumulator l = s + t.
+// With S >= 5 two more sub-passes (phase B) issue the products of levels 4 and 5 into
+// accumulators 2 and 3:
+//   sub-pass 1: stages (A3, B1), (A4, B2), (A2, B0) [, (A5, -)]
+//   sub-pass 2: stages (A1, B4), (A0, B3) [, (A2, B5)]
+// so that no K block needs more than four 24 KB stages.  Stages are loaded in the
+// order in which their last products are issued, and each goes back to the producer
+// right after its own last product: eight stages hold two K blocks, so a stage freed
+// only with its whole K block came back a copy's latency late.
 struct Prod {
     int a, b, acc;   // stage holding the A slice, stage holding the B slice, accumulator
 };
@@ -63,23 +65,42 @@ __host__ __device__ constexpr int sched_nst(int S, int sp) {
     return sp == 0 ? (S < 4 ? S : 4) : sp == 1 ? (S == 6 ? 4 : 3) : (S == 6 ? 3 : 2);
 }
 __host__ __device__ constexpr int sched_sa(int S, int sp, int st) {
-    return sp == 0 ? st : sp == 1 ? 2 + st : st;
+    constexpr int a1[4] = {3, 4, 2, 5}, a2[3] = {1, 0, 2};
+    return sp == 0 ? sched_nst(S, 0) - 1 - st : sp == 1 ? a1[st] : a2[st];
 }
 __host__ __device__ constexpr int sched_sb(int S, int sp, int st) {
-    return sp == 0 ? st : sp == 1 ? (st < 3 ? st : -1) : 3 + st;
+    constexpr int b1[4] = {1, 2, 0, -1}, b2[3] = {4, 3, 5};
+    return sp == 0 ? sched_nst(S, 0) - 1 - st : sp == 1 ? b1[st] : b2[st];
 }
 __host__ __device__ constexpr int sched_nprod(int S, int sp) {
     return sp == 0 ? (S >= 4 ? 10 : S == 3 ? 6 : 3) : sp == 1 ? (S == 6 ? 6 : 3) : (S == 6 ? 5 : 2);
 }
 __host__ __device__ constexpr Prod sched_prod(int S, int sp, int pr) {
-    // sub-pass 0: (s, t) of level l in order l = 0, 1, 2, 3; stages hold slice s.
-    constexpr int s0[10] = {0, 0, 1, 0, 1, 2, 0, 1, 2, 3}, t0[10] = {0, 1, 0, 2, 1, 0, 3, 2, 1, 0};
-    constexpr int l0[10] = {0, 1, 1, 2, 2, 2, 3, 3, 3, 3};
-    // sub-pass 1 (stages A2..A5 / B0..B2): (2,2) (3,1) (4,0) -> level 4; (3,2) (4,1) (5,0) -> level 5
-    constexpr int a1[6] = {0, 1, 2, 1, 2, 3}, b1[6] = {2, 1, 0, 2, 1, 0}, c1[6] = {2, 2, 2, 3, 3, 3};
-    // sub-pass 2 (stages A0..A2 / B3..B5): (0,4) (1,3) -> level 4; (0,5) (1,4) (2,3) -> level 5
-    constexpr int a2[5] = {0, 1, 0, 1, 2}, b2[5] = {1, 0, 2, 1, 0}, c2[5] = {2, 2, 3, 3, 3};
-    return sp == 0 ? Prod{s0[pr], t0[pr], l0[pr]} : sp == 1 ? Prod{a1[pr], b1[pr], c1[pr]} : Prod{a2[pr], b2[pr], c2[pr]};
+    // The products as slices (s, t), highest slices first: level l = s + t.
+    //   sub-pass 0 (four slices; fewer skip the leading ones): accumulator l
+    constexpr int s0[10] = {0, 3, 0, 1, 2, 2, 0, 1, 1, 0}, t0[10] = {3, 0, 2, 2, 1, 0, 1, 1, 0, 0};
+    //   sub-pass 1: levels 4, 5 into accumulators 2, 3; five slices have level 4 only
+    constexpr int s1[6] = {3, 3, 4, 2, 4, 5}, t1[6] = {1, 2, 1, 2, 0, 0};
+    constexpr int s15[3] = {3, 2, 4}, t15[3] = {1, 2, 0};
+    //   sub-pass 2
+    constexpr int s2[5] = {0, 0, 1, 1, 2}, t2[5] = {5, 4, 4, 3, 3};
+    constexpr int s25[2] = {0, 1}, t25[2] = {4, 3};
+    const int k = sp == 0 ? pr + 10 - sched_nprod(S, 0) : pr;
+    const int s = sp == 0 ? s0[k] : sp == 1 ? (S == 6 ? s1[k] : s15[k]) : (S == 6 ? s2[k] : s25[k]);
+    const int t = sp == 0 ? t0[k] : sp == 1 ? (S == 6 ? t1[k] : t15[k]) : (S == 6 ? t2[k] : t25[k]);
+    Prod q{0, 0, sp == 0 ? s + t : s + t - 2};
+    for (int st = 0; st < sched_nst(S, sp); ++st) {
+        if (sched_sa(S, sp, st) == s) q.a = st;
+        if (sched_sb(S, sp, st) == t) q.b = st;
+    }
+    return q;
+}
+// The last product of the sub-pass that reads stage st.
+__host__ __device__ constexpr int sched_last(int S, int sp, int st) {
+    int last = 0;
+    for (int pr = 0; pr < sched_nprod(S, sp); ++pr)
+        if (sched_prod(S, sp, pr).a == st || sched_prod(S, sp, pr).b == st) last = pr;
+    return last;
 }
 // The first product into an accumulator within its phase starts it (accumulate = 0).
 __host__ __device__ constexpr bool sched_first(int S, int sp, int pr) {
@@ -201,38 +222,40 @@ __device__ __forceinline__ bool produce_subpass(const XsParams &p, XsSmemTail &t
     return true;
 }
 
-// MMA issuer: one sub-pass of a tile.  Every product is four K = 16 instructions
+// MMA warp (all lanes): one sub-pass of a tile.  Every product is four K = 16 instructions
 // (M = 256, N = 128) into the accumulator of its level.
 template <int S, int SP>
 __device__ __forceinline__ bool mma_subpass(const XsParams &p, XsSmemTail &tl, uint8_t *stages, unsigned int &idx,
                                             uint32_t tmem_base, const volatile int *abort) {
     constexpr int NST = sched_nst(S, SP), NP = sched_nprod(S, SP);
     const uint32_t idesc = idesc_f16_mn(0u, XS_TILE_M, XS_TILE_N);
+    const uint32_t stage0_lo = sdesc_lo(smem_u32(stages));
     const int nkb = p.np / TC_BK;
     for (int kb = 0; kb < nkb; ++kb) {
         uint32_t sad[NST];
 #pragma unroll
         for (int st = 0; st < NST; ++st) {
             const uint32_t j = idx + st, slot = j % XS_RING;
-            if (!mbar_wait(&tl.full[slot], (j / XS_RING) & 1u, abort, p.timeout_ns, p.err)) return false;
-            sad[st] = smem_u32(stages + (size_t)slot * XS_STAGE_BYTES);
+            if (!mbar_wait_warp(&tl.full[slot], (j / XS_RING) & 1u, abort, p.timeout_ns, p.err)) return false;
+            sad[st] = stage0_lo + slot * (XS_STAGE_BYTES >> 4);
         }
         tc_fence_after();
 #pragma unroll
         for (int pr = 0; pr < NP; ++pr) {
             const Prod q = sched_prod(S, SP, pr);
             const bool first = sched_first(S, SP, pr);
-            const uint32_t a = sad[q.a], b = sad[q.b] + XS_A_BYTES;
+            const uint32_t a = sad[q.a], b = sad[q.b] + (XS_A_BYTES >> 4);
             const uint32_t d = tmem_base + (uint32_t)q.acc * XS_TILE_N;
 #pragma unroll
             for (int k = 0; k < TC_BK / 16; ++k)
-                umma_f16<2>(d, sdesc_sw128(a + k * 32), sdesc_sw128(b + k * 32), idesc,
+                umma_f16<2>(d, a + 2 * k, b + 2 * k, idesc,
                             (first && kb == 0 && k == 0) ? 0u : 1u);
-        }
 #pragma unroll
-        for (int st = 0; st < NST; ++st) umma_commit<2>(&tl.empty[(idx + st) % XS_RING]);
+            for (int st = 0; st < NST; ++st)
+                if (sched_last(S, SP, st) == pr) umma_commit<2>(&tl.empty[(idx + st) % XS_RING]);
+        }
         idx += NST;
-        *(volatile unsigned int *)&tl.consumed = idx;
+        if ((threadIdx.x & 31) == 0) *(volatile unsigned int *)&tl.consumed = idx;
     }
     return true;
 }
@@ -304,12 +327,12 @@ __global__ void __launch_bounds__(XS_THREADS, 1) k_exact_product(const __grid_co
         }
     } else if (warp == 1) {
         // ------------------------------- MMA issuer -------------------------------
-        if (lane == 0 && leader) {
+        if (leader) {
             unsigned int idx = 0;
             int it = 0;
             bool ok = true;
             for (int g = cluster_id; g < p.ntiles; g += nclusters, ++it) {
-                if (!mbar_wait(&tl.teb, (uint32_t)(it & 1) ^ 1u, abort, p.timeout_ns, p.err)) {
+                if (!mbar_wait_warp(&tl.teb, (uint32_t)(it & 1) ^ 1u, abort, p.timeout_ns, p.err)) {
                     ok = false;
                     break;
                 }
@@ -322,7 +345,7 @@ __global__ void __launch_bounds__(XS_THREADS, 1) k_exact_product(const __grid_co
                 if constexpr (PHASE_B) {
                     // Levels 0..3 complete: the epilogue folds them into int64 words in
                     // accumulators 0 and 1 and frees 2 and 3 for levels 4 and 5.
-                    if (!mbar_wait(&tl.tea, (uint32_t)(it & 1), abort, p.timeout_ns, p.err)) {
+                    if (!mbar_wait_warp(&tl.tea, (uint32_t)(it & 1), abort, p.timeout_ns, p.err)) {
                         ok = false;
                         break;
                     }

@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(SIMT_THREADS, TMAX == 128 ? 2 : 4) k_simt_pers
                   "staging of every side the launch runs");
     static_assert(sizeof(sm.stage) >= (4 * MAX_BATCH + 4 * (SIMT_THREADS / 32)) * sizeof(double),
                   "round sums reuse the staging buffers");
-    if (threadIdx.x == 0) round_ctl_init(rc, p);
+    if (threadIdx.x == 0) round_ctl_init(rc, p, p.inst);
     __syncthreads();
     unsigned int target = 0;
     bool first = true;

@@ -13,8 +13,8 @@
 //               X_{(K-1)s} (with FP32 masters in ckf), slots K..K+s-2 the others
 //               by n mod s; the reverse sweep recomputes a segment's layers from
 //               its kept X into those slots (FP32 ping-pong rf).
-//   part[3]     FP64 partials per tile, by layer n mod 3: Tr X, ||X||_F^2,
-//               ||Y||_F^2 and Tr P (see Part).
+//   part[3]     FP64 partials, by layer n mod 3: Tr X, ||X||_F^2, ||Y||_F^2 and Tr P
+//               (see Part).
 //   dataflow schedule (one instance, density mode, tensor cores): three operand
 //               slots; per tile a completion counter (CTAs done, all layers) and a
 //               table of the tiles that write each 256 x 256 block of X.
@@ -36,13 +36,13 @@ namespace sp2i {
 
 constexpr int PAD = 128;            // np is a multiple of this
 constexpr int TC_BM = 128;          // tcgen05 tile rows (UMMA M)
-constexpr int TC_BN = 256;          // tcgen05 tile columns (UMMA N)
+constexpr int TC_BN = 256;          // tcgen05 tile columns (UMMA N) of the wide tiles
 constexpr int TC_BK = 64;           // K block: 64 x 16-bit = one 128-byte swizzle row
-constexpr int TC_STAGES = 4;        // TMA -> MMA pipeline depth
 constexpr int MAPS_PER_SLOT = 5;    // per operand slot: loads hi, hi, lo (64 x 128 boxes); stores hi, lo
 constexpr int EPI_BOX_COLS = 16;    // store box: one epilogue warp's chunk of 32 rows x 16 columns
 constexpr int EPI_BOX_ROWS = 32;
-constexpr int TC_THREADS = 320;     // warp 0 TMA, warp 1 MMA, warps 2..9 epilogue (two per SM sub-partition)
+constexpr int TC_THREADS = 352;     // warp 0 TMA, warp 1 MMA, warps 2..9 epilogue (two per SM sub-partition),
+                                    // warp 10 a batch's decisions
 constexpr int SIMT_THREADS = 128;   // FP32 CUDA-core kernel: 8 x 16 threads on a square tile
 constexpr int MAX_BATCH = 128;
 constexpr int MAX_L = SP2_MAX_LAYERS_LIMIT;
@@ -54,7 +54,10 @@ constexpr double STALL_MAX = 1e-2;
 enum Path { PATH_SIMT = 0, PATH_TC = 1 };
 enum Mode { MODE_DENSITY = 0, MODE_RESPONSE = 1, MODE_ADJOINT = 2, MODE_APPLY = 3 };
 
-// Per-tile FP64 partial sums written by the input layer and every square.
+// FP64 partial sums written by the input layer and every square: on the tensor-core
+// path one record per 256 x 256 pair tile and CTA (128 x 256 tile where those are used),
+// whatever tiles the layer itself runs in, so that a layer's sums, and with them every
+// bit of the chain, do not depend on the tile shape.
 struct __align__(16) Part {
     double t;   // Tr X (stored X)
     double q;   // ||X||_F^2 (stored X)
@@ -68,6 +71,8 @@ struct LayerStatDev {
     double alpha;
 };
 
+constexpr unsigned int FLOW_STOPPED = 0x7FFFFFFFu;
+
 struct InstCtl {
     double eps_min, eps_max, band_energy, trace_D;
     double y_scale;                          // power of two applied to the Y stream
@@ -76,18 +81,19 @@ struct InstCtl {
     unsigned long long ymax_key;
     int nonfinite, status, layers, stop_reason;
     int final_x, final_y, init_parts, degenerate;
-    // Round schedule of a density batch: the CTA that completes an instance's last
-    // tile of layer n sums the layer's partial records (the same fixed order as
-    // every CTA's own sum) and publishes them here, tagged with n.
-    unsigned int psum_done;                  // CTA-tile completions over all layers
-    int psum_n;                              // layer of psum (0: none yet)
-    double psum[4];
+    // Dataflow schedule of a batch: epilogue-warp completions of the instance's tiles over
+    // all layers, and the latest decision as its owner CTA publishes it (flow_seq = layer
+    // + 1, FLOW_STOPPED once the chain has stopped; written last).
+    unsigned int flow_done, flow_seq;
+    int flow_flip;
+    float flow_cf, flow_alpha, pad_flow;
     LayerStatDev stat[MAX_L + 1];
 };
 
 struct InstDesc {
     int n, np, ntiles, tile_off;      // tiles: this instance's slice of the tile table
-    int parts;                        // partial records per layer (tiles x CTAs per tile)
+    int parts;                        // partial records per layer
+    int unit_off, pad_unit;           // narrow tiles: the pair tiles of the records in the tile table
     int kwave;                        // tensor-core path: tiles the device runs at once; tile t walks K
                                       // upward when (t / kwave) is even, downward when odd
     double n_occ;
@@ -105,6 +111,7 @@ struct InstDesc {
     float *yf[2];
     uint16_t *yop;                    // slot s in {0,1}: hi, lo as for xop
     Part *part[3];                    // by layer n mod 3 (three deep for the dataflow schedule)
+    float *pdiag[2];                  // narrow tiles: diagonal of the raw product, by layer parity
     int part_cap, fin_blocks;
     int simt_t, pad_simt;             // FP32 path: tile side (simt_tile_side)
     const CUtensorMap *xmap;          // [nslots_x * MAPS_PER_SLOT]: per slot the K segments' loads op0, op1,
@@ -118,6 +125,11 @@ struct InstDesc {
     InstCtl *ctl;
 };
 
+// Schedules of the tensor-core kernel, each its own kernel: rounds ended by a grid
+// barrier (responses, adjoints, layer application), or no barrier between layers
+// for one density solve and for a batch of them.
+enum Schedule { RUN_ROUNDS = 0, RUN_FLOW = 1, RUN_BATCH = 2 };
+
 struct RunParams {
     InstDesc *inst;
     const int2 *tiles;                // (bi, bj) per tile, per instance slice
@@ -128,12 +140,15 @@ struct RunParams {
     int B, mode, precision, max_layers;
     int test_hook;                    // 1: CTA 0 withholds its first barrier arrival (dataflow:
                                       // its first tile completion)
-    int dataflow;                     // 1: no grid barrier between layers (see the tensor-core kernel)
-    int publish;                      // 1: round schedule of a density batch, sums published per layer
+    int dataflow;                     // schedule of the tensor-core kernel (Schedule)
+    int units;                        // narrow tiles: partial records a layer's statistics pass writes (0: the
+                                      // epilogue writes them)
+    unsigned int *stat_done;          // narrow tiles: records written, all layers
     int nblk;                         // dataflow: 256-row blocks of X (round_up(np, 256) / 256)
-    unsigned int *tile_done;          // dataflow: per tile, CTA completions over all layers
-    unsigned int *layer_done;         // dataflow: CTA-tile completions over all layers
-    const int *blk_src;               // dataflow: [nblk * nblk * 2] tiles writing block (P, Q) of X, -1 none
+    unsigned int *tile_done;          // dataflow: per tile, epilogue-warp completions over all layers
+    unsigned int *layer_done;         // dataflow: epilogue-warp completions over all layers and tiles
+    const int *blk_src;               // dataflow: [nblk * nblk * 2] tiles writing block (P, Q) of X, -1 none;
+                                      // null: a tile waits for the whole previous layer
 };
 
 // Host-side launchers (one translation unit each).
@@ -150,10 +165,11 @@ cudaError_t launch_finalize(InstDesc *inst, int B, int fin_blocks, int mode, cud
 cudaError_t launch_fill_trivial(float *D, int n, float diag_value, cudaStream_t s);
 // FP32 path: `tmax` is the largest tile side of the launch's instances.
 cudaError_t launch_simt_persistent(const RunParams &p, int tmax, int grid, cudaStream_t s);
-cudaError_t launch_tc_persistent(const RunParams &p, int cta_group, int grid, cudaStream_t s);
+cudaError_t launch_tc_persistent(const RunParams &p, int cta_group, int bn, int grid, cudaStream_t s);
 int simt_blocks_per_sm(int tmax);
-int tc_grid_size(int cta_group, int sm_count);
-size_t tc_smem_bytes();
+int tc_grid_size(int cta_group, int bn, int sm_count);
+// Rows of the operand maps' load boxes for tiles of cg CTAs and bn columns.
+inline int tc_box_rows(int cg, int bn) { return bn / cg < 128 ? bn / cg : 128; }
 
 inline int round_up(int a, int b) { return (a + b - 1) / b * b; }
 

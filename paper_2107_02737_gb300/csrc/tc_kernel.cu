@@ -53,20 +53,23 @@ namespace sp2i {
 
 namespace {
 
-// Tile configuration.  CG = 1: one CTA computes a 128 x 256 tile (M = 128 MMAs).
-// CG = 2: a cluster of two CTAs computes a 256 x 256 tile with M = 256 MMAs
-// issued by the even CTA; each CTA loads its own 128 rows of A and 128 of the
-// 256 B rows, so a stage is 32 KB per CTA and six stages fit.
-template <int CG>
+// Tile configuration: 128 CG x BN, BN = 256, 128 or 64.  CG = 2: a cluster of two CTAs
+// computes the tile with M = 256 MMAs issued by the even CTA; each CTA loads its own 128
+// rows of A and half of the B rows.  CG = 1: one CTA, M = 128 MMAs.  An element's
+// products and their order are those of its row and column whatever the tile, so every
+// shape gives the same X; the host picks one by size (narrow_tiles).
+template <int CG, int BN>
 struct Cfg {
-    static constexpr int STAGES = (CG == 2) ? 6 : 4;
+    static constexpr int BOX = BN / CG < 128 ? BN / CG : 128;             // rows per load box (tc_box_rows)
     static constexpr uint32_t A_BYTES = 128 * TC_BK * 2;                   // 16 KB: own 128 rows
-    static constexpr uint32_t B_BYTES = (CG == 2 ? 128 : 256) * TC_BK * 2;  // own B rows
+    static constexpr uint32_t B_BYTES = (BN / CG) * TC_BK * 2;             // own B rows
     static constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
+    static constexpr int STAGES = 196608 / STAGE_BYTES;                    // 4, 6, 8 or 9
     static constexpr uint32_t TX_BYTES = STAGE_BYTES * CG;               // bytes per stage over the pair
     static constexpr int TILE_M = 128 * CG;                              // output rows per tile
+    static constexpr uint32_t TMEM_COLS = 2 * BN;                        // two FP32 accumulators
 };
-constexpr int MAX_STAGES = 6;
+constexpr int MAX_STAGES = 9;
 constexpr int EPI_WARPS = 8;                              // warps 2..9
 constexpr int EPI_CHUNK = 16;                             // accumulator columns per epilogue step
 // Per epilogue warp: the transpose buffer of a chunk (32 x (EPI_CHUNK + 1) words) or
@@ -76,7 +79,6 @@ static_assert(EPI_CHUNK == EPI_BOX_COLS && EPI_BOX_ROWS == 32, "store box = one 
 static_assert(EPI_T_FLOATS >= 32 * (EPI_CHUNK + 1) && EPI_T_FLOATS * 4 >= 2 * EPI_BOX_ROWS * EPI_BOX_COLS * 2 &&
                   (EPI_T_FLOATS * 4) % 128 == 0,
               "epilogue buffer");
-constexpr uint32_t TMEM_COLS = 512;                       // two 128 x 256 FP32 accumulators
 
 struct TcSmemTail {
     uint64_t full[MAX_STAGES];
@@ -88,22 +90,21 @@ struct TcSmemTail {
     uint32_t pad;
     unsigned int issued;             // producer: ring stages this CTA has loaded into
     unsigned int consumed;           // MMA thread (even CTA): stages whose copies it has waited for
-    FF red[EPI_WARPS][4];            // per epilogue warp: the tile's four partials (compensated pairs)
-    double flow_sums[4];             // dataflow: the previous layer's sums
+    FF red[EPI_WARPS][4];            // per epilogue warp: a record's four partials (compensated pairs)
+    double flow_sums[5];             // dataflow: the layer's sums; [4] nonzero: a wait gave up
     RoundCtl rc;
+    InstDesc desc;                   // a lone instance's descriptor (global loads of it would miss L1
+                                     // after every acquire)
 };
 
-constexpr size_t STAGE_AREA = 196608;  // 4 x 48 KB or 6 x 32 KB
-static_assert(Cfg<1>::STAGES * Cfg<1>::STAGE_BYTES <= STAGE_AREA, "stage area");
-static_assert(Cfg<2>::STAGES * Cfg<2>::STAGE_BYTES <= STAGE_AREA, "stage area");
+constexpr size_t STAGE_AREA = 196608;  // 4 x 48 KB, 6 x 32 KB, 8 x 24 KB or 9 x 20 KB
 static_assert(EPI_WARPS * EPI_T_FLOATS * 4 >= 4 * MAX_BATCH * sizeof(double) + MAX_BATCH * sizeof(int),
               "round sums and decisions reuse the epilogue transpose buffers");
 constexpr size_t SMEM_BYTES = 1024 /*alignment slack*/ + STAGE_AREA + (size_t)EPI_WARPS * EPI_T_FLOATS * 4 +
                               sizeof(TcSmemTail);
 
 // Instruction descriptor, kind::f16: FP32 accumulator, A and B of one 16-bit
-// type (0 = FP16, 1 = BF16), both K-major, N = 256, M = 128 * CG.
-__host__ __device__ constexpr uint32_t idesc_f16(uint32_t ab, int m) { return idesc_f16_mn(ab, m, TC_BN); }
+// type (0 = FP16, 1 = BF16), both K-major, M = 128 * CG, N = BN: idesc_f16_mn.
 
 // ---------------------------------------------------------------------------
 // Work description of one tile, identical for the three roles.
@@ -130,8 +131,8 @@ __device__ __forceinline__ void tc_abort(RoundCtl &rc, uint32_t peer_abort) {
 
 __device__ __forceinline__ TileWork describe(const RoundCtl &rc, const RunParams &p, int g) {
     TileWork w;
-    map_tile(rc, p.B, p.inst, g, w.inst, w.job, w.tile);
-    const InstDesc &d = p.inst[w.inst];
+    map_tile(rc, p.B, rc.inst, g, w.inst, w.job, w.tile);
+    const InstDesc &d = rc.inst[w.inst];
     const int2 bt = p.tiles[d.tile_off + w.tile];
     w.bi = bt.x;
     w.bj = bt.y;
@@ -169,12 +170,11 @@ __device__ __forceinline__ TileWork describe(const RoundCtl &rc, const RunParams
     return w;
 }
 
-// Dataflow schedule: tile g of layer r for the producer and the MMA thread (the
+// Dataflow schedule: tile g (at bt) of layer r for the producer and the MMA thread (the
 // layer's sign and offset are not needed there).
-__device__ __forceinline__ TileWork describe_flow(const RunParams &p, int g, int r) {
+__device__ __forceinline__ TileWork describe_flow(const RoundCtl &rc, int g, int2 bt, int r) {
     TileWork w;
-    const InstDesc &d = p.inst[0];
-    const int2 bt = p.tiles[d.tile_off + g];
+    const InstDesc &d = rc.inst[0];
     w.inst = 0;
     w.job = 0;
     w.tile = g;
@@ -193,7 +193,7 @@ __device__ __forceinline__ TileWork describe_flow(const RunParams &p, int g, int
 
 // Dataflow schedule, producer.  A 256-column block kt of the operand row blocks pa
 // and pb of X_n was written by at most four tiles of the previous layer, each done
-// when its counter reaches `target` (CG completions per layer).  The counters are
+// when its counter reaches `target` (EPI_WARPS * CG completions per layer).  The counters are
 // read with relaxed loads one block ahead (flow_peek), so their latency hides under
 // the current block's copies, and re-polled only while a tile is still running;
 // one acquire fence then orders the TMA reads after the tiles' stores.
@@ -208,7 +208,7 @@ __device__ __forceinline__ void flow_peek(const RunParams &p, int pa, int pb, in
 #pragma unroll
     for (int k = 0; k < 4; ++k) v[k] = src[k] < 0 ? 0xFFFFFFFFu : ld_relaxed(p.tile_done + src[k]);
 }
-__device__ __noinline__ bool flow_wait(const RunParams &p, int pa, int pb, int kt, unsigned int target,
+__device__ __noinline__ bool flow_wait_block(const RunParams &p, int pa, int pb, int kt, unsigned int target,
                                        unsigned int (&v)[4], const volatile int *abort) {
     const int *e0 = p.blk_src + (pa * p.nblk + kt) * 2, *e1 = p.blk_src + (pb * p.nblk + kt) * 2;
     const int src[4] = {e0[0], e0[1], e1[0], e1[1]};
@@ -230,68 +230,253 @@ __device__ __noinline__ bool flow_wait(const RunParams &p, int pa, int pb, int k
     return true;
 }
 
-// Dataflow schedule, the eight epilogue warps: wait for every CTA-tile of layer r - 1
-// (`per_layer` completions each), then the same sums in the same order as the
-// barrier schedule (one warp) and the same decision for instance 0.  Returns false
-// when the chain stopped or the launch is stopping.  `sums` is four doubles of
-// shared memory.
-__device__ __noinline__ bool flow_decide(RoundCtl &rc, const RunParams &p, double *sums, int r, int ew, int lane,
-                                         unsigned int per_layer, const volatile int *abort) {
+// Dataflow schedule: wait until a counter (epilogue warps done with a tile of layers
+// 0 .. r - 1, or records written) has reached `target`; false when the launch is
+// stopping or the wait ran out.  Relaxed polls and one acquire load at the end (0.4 us less than a fence).
+__device__ __forceinline__ bool flow_wait(const RunParams &p, const unsigned int *counter, unsigned int target,
+                                          const volatile int *abort) {
+    if (ld_relaxed(counter) < target) {
+        const unsigned long long t0 = global_ns();
+        for (int i = 0; ld_relaxed(counter) < target; ++i) {
+            if ((i & 31) != 31) continue;   // the clock and the flags now and then
+            if (*abort || ld_volatile(p.err) != 0) return false;
+            if (global_ns() - t0 > p.timeout_ns) {
+                set_error(p.err, SP2_ERR_TIMEOUT);
+                return false;
+            }
+            __nanosleep(64);
+        }
+    }
+    return ld_acquire(counter) >= target;
+}
+
+// The eight epilogue warps: one partial record from each warp's compensated pairs, which
+// stay FP32 pairs through the warp and cross-warp sums (FP64 arithmetic is slow on this
+// part); one conversion, written by one thread (epilogue warp 0, lane 0).
+__device__ __forceinline__ void write_record(FF (&red)[EPI_WARPS][4], Part *out, const FF &ft, const FF &fq,
+                                             const FF &fw, const FF &fp, int ew, int lane) {
+    FF qw = fq;
+    ff_add_ff(qw, fw);
+    const FF r4[4] = {ff_warp_sum(ft), ff_warp_sum(fq), ff_warp_sum(qw), ff_warp_sum(fp)};
+    if (lane == 0)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) red[ew][k] = r4[k];
+    asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32) : "memory");
     if (ew == 0 && lane == 0) {
-        int go = 1;
-        if (r > 0) {
-            const unsigned int target = per_layer * (unsigned int)r;
-            const unsigned long long t0 = global_ns();
-            while (ld_acquire(p.layer_done) < target) {
-                if (*abort || ld_volatile(p.err) != 0) {
-                    go = 0;
-                    break;
-                }
-                if (global_ns() - t0 > p.timeout_ns) {
-                    set_error(p.err, SP2_ERR_TIMEOUT);
-                    go = 0;
-                    break;
-                }
-                __nanosleep(64);
+        FF a4[4] = {red[0][0], red[0][1], red[0][2], red[0][3]};
+        for (int k = 1; k < EPI_WARPS; ++k)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) ff_add_ff(a4[c], red[k][c]);
+        Part s4;
+        s4.t = ff_value(a4[0]);
+        s4.q = ff_value(a4[1]);
+        s4.w = ff_value(a4[2]);
+        s4.p = ff_value(a4[3]);
+        *out = s4;
+    }
+}
+
+// Narrow tiles, the eight epilogue warps: record u of X_n, the sums over the 128 x 256
+// elements that CTA u mod 2 of pair tile u / 2 would own, by the same warps' rows and
+// columns and in the same order as that CTA's epilogue adds them.  X_n comes back from
+// its FP32 master (lower triangle, coalesced across the warp).  The pass runs once the layer's tiles are complete, beside the next layer's copies and
+// MMAs, which need no statistics; only the next epilogue does.
+__device__ __forceinline__ void flow_record(FF (&red)[EPI_WARPS][4], const InstDesc &d, const int2 *units, int u, int n,
+                                         int ew, int lane) {
+    const int np = d.np;
+    const int2 bt = units[u >> 1];
+    const float *X = d.xf[n & 1];
+    const int rw0 = bt.x * 256 + (u & 1) * 128 + ((ew + 2) & 3) * 32, r = rw0 + lane;
+    const int col0 = bt.y * 256 + (ew >> 2) * 128;
+    int j0 = 0, j1 = (rw0 < np) ? 128 / EPI_CHUNK : 0;
+    while (j1 > 0 && col0 + (j1 - 1) * EPI_CHUNK >= np) --j1;
+    while (j0 < j1 && col0 + j0 * EPI_CHUNK + EPI_CHUNK - 1 < rw0) ++j0;
+    FF ft = {0.f, 0.f}, fq = {0.f, 0.f}, fp = {0.f, 0.f}, fw = {0.f, 0.f};
+    // A short loop, three chunks of loads ahead: the pass is bound by instruction fetch
+    // (unrolled over 64 columns it took twice as long) and by the loads' latency.
+    const float pd = (j0 < j1 && r < d.n) ? __ldcg(d.pdiag[n & 1] + r) : 0.0f;
+    const float *p = X + (size_t)(col0 + j0 * EPI_CHUNK) * np + r;
+    const size_t step = (size_t)EPI_CHUNK * np;
+    float x[EPI_CHUNK], y[EPI_CHUNK], z[EPI_CHUNK], u3[EPI_CHUNK];
+    auto load = [&](int j, float (&v)[EPI_CHUNK]) {
+        if (j < j1) {
+#pragma unroll
+            for (int jj = 0; jj < EPI_CHUNK; ++jj) v[jj] = __ldcg(p + (size_t)jj * np);
+        }
+        p += step;
+    };
+    load(j0, x);
+    load(j0 + 1, y);
+    load(j0 + 2, z);
+#pragma unroll 1
+    for (int j = j0; j < j1; ++j) {
+        load(j + 3, u3);
+        const int jd = r - (col0 + j * EPI_CHUNK);   // the diagonal's column in the chunk
+        float xd = 0.0f;
+#pragma unroll
+        for (int jj = 0; jj < EPI_CHUNK; ++jj) {
+            ff_add_sq(fq, jj >= jd ? x[jj] : 0.0f, jj == jd ? 1.0f : 2.0f);
+            if (jj == jd) xd = x[jj];
+        }
+        if (jd >= 0 && jd < EPI_CHUNK) {
+            ff_add(ft, xd);
+            if (r < d.n) {
+                ff_add(fp, pd);
+                ff_add_sq(fw, xd - 0.5f, 1.0f);
+                ff_add_sq(fw, xd, -1.0f);
             }
         }
-        if (ld_volatile(p.err) != 0) go = 0;
-        rc.flow_go = go;
+#pragma unroll
+        for (int jj = 0; jj < EPI_CHUNK; ++jj) {
+            x[jj] = y[jj];
+            y[jj] = z[jj];
+            z[jj] = u3[jj];
+        }
     }
-    asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32) : "memory");
-    if (!rc.flow_go) return false;
-    if (ew == 0) {
-        double a[4];
-        sum_instance_partials(rc, p, 0, lane, a);
-        if (lane == 0)
-            for (int c = 0; c < 4; ++c) sums[c] = a[c];
+    write_record(red, d.part[n % 3] + u, ft, fq, fw, fp, ew, lane);
+}
+
+// Dataflow schedule of a batch.  Every CTA walks the same fixed list of tiles layer
+// after layer, and an instance's tiles start layer n as soon as its own layer n - 1 is
+// complete and decided, whatever the others do: no barrier, and a pair's remainder of one
+// round overlaps the next.  (Every wait is for a list entry a whole round earlier, so the
+// first unfinished entry never waits.)  The decisions of instance i are taken by one
+// CTA, i mod grid, in a warp of its own, and published in the instance's control block.
+
+// 1: instance `ctl` runs layer r, 0: its chain has stopped, -1: the launch is stopping.
+__device__ __forceinline__ int flow_wait_instance(const RunParams &p, const InstCtl *ctl, int r,
+                                                  const volatile int *abort) {
+    unsigned int seq = ld_relaxed(&ctl->flow_seq);
+    if (seq < (unsigned int)r + 1u) {
+        const unsigned long long t0 = global_ns();
+        for (int i = 0; (seq = ld_relaxed(&ctl->flow_seq)) < (unsigned int)r + 1u; ++i) {
+            if ((i & 31) != 31) continue;
+            if (*abort || ld_volatile(p.err) != 0) return -1;
+            if (global_ns() - t0 > p.timeout_ns) {
+                set_error(p.err, SP2_ERR_TIMEOUT);
+                return -1;
+            }
+            __nanosleep(64);
+        }
+    }
+    return ld_acquire(&ctl->flow_seq) == FLOW_STOPPED ? 0 : 1;
+}
+
+// One warp: sums and decides for instances blockIdx.x, blockIdx.x + gridDim.x, ... until
+// all of them have stopped.
+template <int CG>
+__device__ __noinline__ void flow_owner(RoundCtl &rc, const RunParams &p, int lane, const volatile int *abort) {
+    int left = 0;
+    for (int i = blockIdx.x; i < p.B; i += gridDim.x) ++left;
+    unsigned long long t0 = global_ns();
+    for (bool first = true; left > 0; first = false) {
+        bool progress = false;
+        for (int i = blockIdx.x; i < p.B; i += gridDim.x) {
+            if (!first && !rc.active[i]) continue;
+            InstCtl *ctl = rc.inst[i].ctl;
+            const int n = rc.layer[i] + (rc.ran[i] ? 1 : 0);   // the layer whose records come next
+            int ready = 1;
+            if (!first && lane == 0) {
+                const unsigned int target = (unsigned int)(EPI_WARPS * CG * rc.inst[i].ntiles) * (unsigned int)n;
+                ready = (ld_relaxed(&ctl->flow_done) >= target && ld_acquire(&ctl->flow_done) >= target) ? 1 : 0;
+            }
+            if (!__shfl_sync(0xffffffffu, ready, 0)) continue;
+            double sums[4] = {0.0, 0.0, 0.0, 0.0};
+            if (rc.active[i]) sum_layer_partials(rc.inst[i], n, lane, sums);
+            int go = 0;
+            if (lane == 0) {
+                go = decide_instance(rc, p, sums, i, true) > 0 ? 1 : 0;
+                ctl->flow_flip = rc.choice[i] == SP2_CHOICE_FLIP;
+                ctl->flow_cf = (float)rc.coff[i];
+                ctl->flow_alpha = rc.alpha[i];
+                asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(&ctl->flow_seq),
+                             "r"(go ? (unsigned int)n + 1u : FLOW_STOPPED)
+                             : "memory");
+            }
+            __syncwarp();
+            progress = true;
+            if (!__shfl_sync(0xffffffffu, go, 0)) --left;
+        }
+        if (progress) {
+            t0 = global_ns();
+            continue;
+        }
+        int stop = 0;
+        if (lane == 0) {
+            if (*abort || ld_volatile(p.err) != 0) stop = 1;
+            else if (global_ns() - t0 > p.timeout_ns) {
+                set_error(p.err, SP2_ERR_TIMEOUT);
+                stop = 1;
+            }
+        }
+        if (__shfl_sync(0xffffffffu, stop, 0)) return;
+        __nanosleep(100);
+    }
+}
+
+// Dataflow schedule, the eight epilogue warps: wait for layer r - 1 (with narrow tiles,
+// compute this CTA's record of it and wait for the other CTAs'), the sums of its records
+// in a fixed order (a warp per value) and the decision for instance 0; one barrier hands it to
+// the others (flow_go by parity: the next decision cannot pass this one's readers, who
+// arrive at its barrier first).  Returns false when the chain stopped or the launch is
+// stopping.
+template <bool NARROW>
+__device__ __forceinline__ bool flow_decide(RoundCtl &rc, FF (&red)[EPI_WARPS][4], double *sums, const RunParams &p,
+                                         int r, int ew, int lane, unsigned int per_layer, const volatile int *abort) {
+    if (!NARROW && !p.blk_src) {
+        // Wide tiles in one wave: one warp does it all while the others wait at the
+        // barrier (51.5 against 48.2 us per layer at N = 2304 with the steps below, which
+        // win where tiles come in several waves: 121.0 against 122.6 us at N = 4096).
+        if (ew == 0) {
+            int go = 1;
+            if (lane == 0 && r > 0) go = flow_wait(p, p.layer_done, per_layer * (unsigned int)r, abort) ? 1 : 0;
+            go = __shfl_sync(0xffffffffu, go, 0);
+            double a[4];
+            if (go) sum_layer_partials(rc.inst[0], r, lane, a);
+            if (lane == 0) {
+                if (ld_volatile(p.err) != 0) go = 0;
+                if (go) go = decide_instance(rc, p, a, 0, blockIdx.x == 0) > 0 ? 1 : 0;
+                rc.flow_go[r & 1] = go;
+            }
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32) : "memory");
+        return rc.flow_go[r & 1] != 0;
+    }
+    // One thread of a CTA polls (more of them slowed the increments themselves).
+    const bool unit = r > 0 && p.units > 0 && (int)blockIdx.x < p.units;
+    if (r > 0 && (unit || p.units == 0)) {
+        if (ew == 0 && lane == 0 && !flow_wait(p, p.layer_done, per_layer * (unsigned int)r, abort)) sums[4] = 1.0;
+        asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32) : "memory");
+    }
+    // (An aborting launch goes through the same barriers, with whatever X holds.)
+    if (unit) flow_record(red, rc.inst[0], p.tiles + rc.inst[0].unit_off, blockIdx.x, r, ew, lane);
+    if (r > 0 && p.units > 0) {
+        if (ew == 0 && lane == 0) {
+            if (unit) {
+                __threadfence();
+                atomicAdd(p.stat_done, 1u);
+            }
+            if (!flow_wait(p, p.stat_done, (unsigned int)p.units * (unsigned int)r, abort)) sums[4] = 1.0;
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32) : "memory");
+    }
+    if (ew < 4) {   // warp c sums value c of the records
+        const double a = sum_layer_value(rc.inst[0], r, ew, lane);
+        if (lane == 0) sums[ew] = a;
     }
     asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32) : "memory");
     if (ew == 0 && lane == 0) {
-        const int width = decide_instance(rc, p, sums, 0, blockIdx.x == 0);
-        rc.prefix[0] = 0;
-        rc.prefix[1] = width;
-        rc.total = width;
+        int go = sums[4] == 0.0 && ld_volatile(p.err) == 0;
+        if (go) go = decide_instance(rc, p, sums, 0, blockIdx.x == 0) > 0 ? 1 : 0;
+        rc.flow_go[r & 1] = go;
     }
     asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32) : "memory");
-    return rc.total > 0;
+    return rc.flow_go[r & 1] != 0;
 }
 
-// Element jj of a lane's chunk row into the packed column pairs of its hi and lo boxes.
-__device__ __forceinline__ void pack_pair(uint32_t (&hp)[EPI_CHUNK / 2], uint32_t (&lp)[EPI_CHUNK / 2], int jj,
-                                          uint16_t a1, uint16_t a2) {
-    if (jj & 1) {
-        hp[jj >> 1] |= (uint32_t)a1 << 16;
-        lp[jj >> 1] |= (uint32_t)a2 << 16;
-    } else {
-        hp[jj >> 1] = a1;
-        lp[jj >> 1] = a2;
-    }
-}
-
-template <int PREC, int CG>
+template <int PREC, int CG, int BN, int SCHED>
 __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_constant__ RunParams p) {
-    using C = Cfg<CG>;
+    using C = Cfg<CG, BN>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t *stages = smem;
@@ -317,21 +502,27 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
         mbar_init(&tl.drain, 1);
         tl.issued = 0;
         tl.consumed = 0;
+        tl.flow_sums[4] = 0.0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        round_ctl_init(rc, p);
+        if (p.B == 1) tl.desc = p.inst[0];
+        round_ctl_init(rc, p, p.B == 1 ? &tl.desc : p.inst);
+        if (SCHED == RUN_BATCH) {
+            rc.prefix[0] = 0;
+            for (int i = 0; i < p.B; ++i) rc.prefix[i + 1] = rc.prefix[i] + p.inst[i].ntiles;
+        }
     }
     if (warp == 1) {
         if (CG == 2) {
             asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                              smem_u32(&tl.tmem_base)),
-                         "r"(TMEM_COLS)
+                         "r"(C::TMEM_COLS)
                          : "memory");
             asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
         } else {
             asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                              smem_u32(&tl.tmem_base)),
-                         "r"(TMEM_COLS)
+                         "r"(C::TMEM_COLS)
                          : "memory");
             asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
         }
@@ -357,7 +548,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
     int pend[MAX_STAGES];               // producer: parity + 1 of a load not yet released
     for (int s = 0; s < MAX_STAGES; ++s) pend[s] = 0;
     unsigned int issued = 0, consumed = 0;   // producer / MMA thread: ring stages so far
-    const uint32_t idesc = idesc_f16(PREC == SP2_BF16_SPLIT ? 1u : 0u, C::TILE_M);
+    const uint32_t stage0_lo = sdesc_lo(smem_u32(stages));
+    const uint32_t idesc = idesc_f16_mn(PREC == SP2_BF16_SPLIT ? 1u : 0u, C::TILE_M, BN);
 
     // ---------- per-tile work of the three roles (both schedules below) ----------
     // Producer: every K block of tile w into the ring.  In the dataflow schedule a
@@ -368,36 +560,46 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
         // Dataflow: the column block checked last, the one peeked ahead and its counters.
         int df_kt = -1, df_next = -1;
         unsigned int df_v[4] = {0u, 0u, 0u, 0u};
-        bool df_ready = !p.dataflow || w.n == 0 || df_round == w.n;
+        bool df_ready = SCHED != RUN_FLOW || w.n == 0 || df_round == w.n;
+        if (!df_ready && !p.blk_src) {
+            // One wave of tiles or little more: the layer's tiles end together.
+            if (!flow_wait(p, p.layer_done, (unsigned int)(EPI_WARPS * CG * rc.inst[0].ntiles * w.n), abort)) {
+                tc_abort<CG>(rc, peer_abort);
+                return;
+            }
+            df_round = w.n;
+            df_ready = true;
+            asm volatile("fence.proxy.async.global;" ::: "memory");
+        }
         if (!df_ready) {
-            if (ld_relaxed(p.layer_done) >= (unsigned int)(CG * p.inst[0].ntiles * w.n)) {
+            if (ld_relaxed(p.layer_done) >= (unsigned int)(EPI_WARPS * CG * rc.inst[0].ntiles * w.n)) {
                 df_round = w.n;   // every tile of the previous layer is done
                 df_ready = true;
             } else {
                 // Or every tile that wrote this tile's two operand row blocks is: one pass
                 // of relaxed loads (all in flight together), no per-block checks then.
                 const int pa = (w.bi * C::TILE_M + (int)rank * 128) / 256, pb = w.bj;
-                const int nb = (p.inst[0].np + 255) / 256;
+                const int nb = (rc.inst[0].np + 255) / 256;
                 unsigned int mn = 0xFFFFFFFFu;
                 for (int kt = 0; kt < nb; ++kt) {
                     unsigned int v[4];
                     flow_peek(p, pa, pb, kt, v);
                     mn = min(mn, min(min(v[0], v[1]), min(v[2], v[3])));
                 }
-                df_ready = mn >= (unsigned int)(CG * w.n);
+                df_ready = mn >= (unsigned int)(EPI_WARPS * CG * w.n);
             }
             if (df_ready) {
                 asm volatile("fence.acq_rel.gpu;" ::: "memory");
                 asm volatile("fence.proxy.async.global;" ::: "memory");
             }
         }
-        const InstDesc &d = p.inst[w.inst];
+        const InstDesc &d = rc.inst[w.inst];
         const int nkb = d.np / TC_BK;
         // Successive waves of tiles walk K in opposite directions, so that a
         // wave starts on the K blocks the previous one left in L2.
         const bool kdown = ((w.tile / d.kwave) & 1) != 0;
         const int row_a = w.bi * C::TILE_M + (int)rank * 128;
-        const int row_b = w.bj * TC_BN + (CG == 2 ? (int)rank * 128 : 0);
+        const int row_b = w.bj * BN + (CG == 2 ? (int)rank * (BN / 2) : 0);
         // Square tiles: each K block in two consecutive ring slots, (hi, hi) then
         // (lo, lo), which feed all three products.  Response tiles: the six
         // segments one after another, one K block per slot.
@@ -426,7 +628,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
                 df_kt = kx / 256;
                 const int pa = row_a / 256, pb = row_b / 256;
                 if (df_next != df_kt) flow_peek(p, pa, pb, df_kt, df_v);
-                if (!flow_wait(p, pa, pb, df_kt, (unsigned int)(CG * w.n), df_v, abort)) {
+                if (!flow_wait_block(p, pa, pb, df_kt, (unsigned int)(EPI_WARPS * CG * w.n), df_v, abort)) {
                     tc_abort<CG>(rc, peer_abort);
                     break;
                 }
@@ -445,15 +647,20 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
             uint8_t *sa = stages + (size_t)stage * C::STAGE_BYTES;
             if (CG == 1) {
                 mbar_expect_tx(&tl.full[stage], C::TX_BYTES);
-                tma_load_2d(sa, am, kx, row_a, &tl.full[stage]);
-                tma_load_2d(sa + C::A_BYTES, bm, kx, row_b, &tl.full[stage]);
-                tma_load_2d(sa + C::A_BYTES + C::B_BYTES / 2, bm, kx, row_b + 128, &tl.full[stage]);
+#pragma unroll
+                for (int q = 0; q < 128; q += C::BOX)
+                    tma_load_2d(sa + q * (TC_BK * 2), am, kx, row_a + q, &tl.full[stage]);
+#pragma unroll
+                for (int q = 0; q < BN; q += C::BOX)
+                    tma_load_2d(sa + C::A_BYTES + q * (TC_BK * 2), bm, kx, row_b + q, &tl.full[stage]);
             } else {
                 // Both CTAs' bytes complete on the even CTA's barrier.
                 if (leader) mbar_expect_tx(&tl.full[stage], C::TX_BYTES);
                 const uint32_t fb = lead_full0 + stage * 8u;
-                tma_load_2d_pair(sa, am, kx, row_a, fb);
-                tma_load_2d_pair(sa + C::A_BYTES, bm, kx, row_b, fb);
+#pragma unroll
+                for (int q = 0; q < 128; q += C::BOX)
+                    tma_load_2d_pair(sa + q * (TC_BK * 2), am, kx, row_a + q, fb);
+                tma_load_2d_pair(sa + C::A_BYTES, bm, kx, row_b, fb);   // BN / 2 rows: one box
             }
             pend[stage] = (int)phase + 1;
             *(volatile unsigned int *)&tl.issued = ++issued;
@@ -463,112 +670,57 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
             }
         }
     };
-    // MMA issuer: tile w's products into the next accumulator; false when a wait
-    // gave up (the launch is stopping).
+    // MMA warp (the leader CTA's, all lanes): tile w's products into the next
+    // accumulator; false when a wait gave up (the launch is stopping).
+    // One ring slot: its operands' low descriptor word, or 0 when the wait gave up.
+    auto mma_slot = [&](uint32_t &slot) -> uint32_t {
+        slot = stage;
+        if (!mbar_wait_warp(&tl.full[stage], phase, abort, p.timeout_ns, p.err)) {
+            tc_abort<CG>(rc, peer_abort);
+            return 0;
+        }
+        ++consumed;
+        if (lane == 0) *(volatile unsigned int *)&tl.consumed = consumed;
+        if (++stage == C::STAGES) {
+            stage = 0;
+            phase ^= 1u;
+        }
+        return stage0_lo + slot * (C::STAGE_BYTES >> 4);
+    };
     auto mma_tile = [&](const TileWork &w) -> bool {
-        const InstDesc &d = p.inst[w.inst];
-        if (!mbar_wait(&tl.tempty[acc], acc_phase ^ 1u, abort, p.timeout_ns, p.err)) {
+        if (!mbar_wait_warp(&tl.tempty[acc], acc_phase ^ 1u, abort, p.timeout_ns, p.err)) {
             tc_abort<CG>(rc, peer_abort);
             return false;
         }
         tc_fence_after();
-        const uint32_t d_tmem = tmem_base + acc * TC_BN;
+        const uint32_t d_tmem = tmem_base + acc * BN;
+        constexpr uint32_t B_OFF = C::A_BYTES >> 4;
         bool ok = true;
-        if (!w.resp) {
-            // Square: per K block the (hi, hi) and (lo, lo) slots, then hi lo, lo hi
-            // (the small cross terms first) and hi hi.
-            for (int kb = 0; kb < d.np / TC_BK; ++kb) {
-                uint32_t sh, sl;
-                const uint32_t st_h = stage;
-                if (!mbar_wait(&tl.full[stage], phase, abort, p.timeout_ns, p.err)) {
-                    tc_abort<CG>(rc, peer_abort);
-                    ok = false;
-                    break;
-                }
-                *(volatile unsigned int *)&tl.consumed = ++consumed;
-                sh = smem_u32(stages + (size_t)stage * C::STAGE_BYTES);
-                if (++stage == C::STAGES) {
-                    stage = 0;
-                    phase ^= 1u;
-                }
-                const uint32_t st_l = stage;
-                if (!mbar_wait(&tl.full[stage], phase, abort, p.timeout_ns, p.err)) {
-                    tc_abort<CG>(rc, peer_abort);
-                    ok = false;
-                    break;
-                }
-                *(volatile unsigned int *)&tl.consumed = ++consumed;
-                sl = smem_u32(stages + (size_t)stage * C::STAGE_BYTES);
-                if (++stage == C::STAGES) {
-                    stage = 0;
-                    phase ^= 1u;
-                }
-                tc_fence_after();
-#pragma unroll
-                for (int k = 0; k < TC_BK / 16; ++k)   // hi x lo
-                    umma_f16<CG>(d_tmem, sdesc_sw128(sh + k * 32), sdesc_sw128(sl + C::A_BYTES + k * 32),
-                                 idesc, (kb | k) != 0 ? 1u : 0u);
-#pragma unroll
-                for (int k = 0; k < TC_BK / 16; ++k)   // lo x hi
-                    umma_f16<CG>(d_tmem, sdesc_sw128(sl + k * 32), sdesc_sw128(sh + C::A_BYTES + k * 32),
-                                 idesc, 1u);
-#pragma unroll
-                for (int k = 0; k < TC_BK / 16; ++k)   // hi x hi
-                    umma_f16<CG>(d_tmem, sdesc_sw128(sh + k * 32), sdesc_sw128(sh + C::A_BYTES + k * 32),
-                                 idesc, 1u);
-                umma_commit<CG>(&tl.empty[st_h]);
-                umma_commit<CG>(&tl.empty[st_l]);
+        // Per K block, a square: the (hi, hi) and (lo, lo) slots, then hi lo, lo hi (the
+        // small cross terms first) and hi hi.  A response: the slots (X hi, Y hi),
+        // (X lo, Y lo) for X Y^T, released as soon as those products are issued, then
+        // (Y hi, X hi), (Y lo, X lo) for Y X^T; cross terms before hi x hi in each.
+        const int nslots = rc.inst[w.inst].np / TC_BK * (w.resp ? 2 : 1);
+        for (int kb = 0; kb < nslots; ++kb) {
+            uint32_t st_h, st_l;
+            const uint32_t sh = mma_slot(st_h);
+            const uint32_t sl = sh ? mma_slot(st_l) : 0u;
+            if (!sl) {
+                ok = false;
+                break;
             }
-        }
-        if (w.resp) {
-            // Response: per K block the slots (X hi, Y hi), (X lo, Y lo) for X Y^T,
-            // released as soon as those products are issued, then (Y hi, X hi),
-            // (Y lo, X lo) for Y X^T; cross terms before hi x hi in each.
-            for (int kb = 0; ok && kb < d.np / TC_BK; ++kb) {
-#pragma unroll 1
-                for (int pr = 0; pr < 2; ++pr) {
-                    const uint32_t st_h = stage;
-                    if (!mbar_wait(&tl.full[stage], phase, abort, p.timeout_ns, p.err)) {
-                        tc_abort<CG>(rc, peer_abort);
-                        ok = false;
-                        break;
-                    }
-                    *(volatile unsigned int *)&tl.consumed = ++consumed;
-                    const uint32_t sh = smem_u32(stages + (size_t)stage * C::STAGE_BYTES);
-                    if (++stage == C::STAGES) {
-                        stage = 0;
-                        phase ^= 1u;
-                    }
-                    const uint32_t st_l = stage;
-                    if (!mbar_wait(&tl.full[stage], phase, abort, p.timeout_ns, p.err)) {
-                        tc_abort<CG>(rc, peer_abort);
-                        ok = false;
-                        break;
-                    }
-                    *(volatile unsigned int *)&tl.consumed = ++consumed;
-                    const uint32_t sl = smem_u32(stages + (size_t)stage * C::STAGE_BYTES);
-                    if (++stage == C::STAGES) {
-                        stage = 0;
-                        phase ^= 1u;
-                    }
-                    tc_fence_after();
+            tc_fence_after();
 #pragma unroll
-                    for (int k = 0; k < TC_BK / 16; ++k)   // A hi x B lo
-                        umma_f16<CG>(d_tmem, sdesc_sw128(sh + k * 32),
-                                     sdesc_sw128(sl + C::A_BYTES + k * 32), idesc,
-                                     (kb | pr | k) != 0 ? 1u : 0u);
+            for (int k = 0; k < TC_BK / 16; ++k)   // hi x lo
+                umma_f16<CG>(d_tmem, sh + 2 * k, sl + B_OFF + 2 * k, idesc, (kb | k) != 0 ? 1u : 0u);
 #pragma unroll
-                    for (int k = 0; k < TC_BK / 16; ++k)   // A lo x B hi
-                        umma_f16<CG>(d_tmem, sdesc_sw128(sl + k * 32),
-                                     sdesc_sw128(sh + C::A_BYTES + k * 32), idesc, 1u);
+            for (int k = 0; k < TC_BK / 16; ++k)   // lo x hi
+                umma_f16<CG>(d_tmem, sl + 2 * k, sh + B_OFF + 2 * k, idesc, 1u);
 #pragma unroll
-                    for (int k = 0; k < TC_BK / 16; ++k)   // A hi x B hi
-                        umma_f16<CG>(d_tmem, sdesc_sw128(sh + k * 32),
-                                     sdesc_sw128(sh + C::A_BYTES + k * 32), idesc, 1u);
-                    umma_commit<CG>(&tl.empty[st_h]);
-                    umma_commit<CG>(&tl.empty[st_l]);
-                }
-            }
+            for (int k = 0; k < TC_BK / 16; ++k)   // hi x hi
+                umma_f16<CG>(d_tmem, sh + 2 * k, sh + B_OFF + 2 * k, idesc, 1u);
+            umma_commit<CG>(&tl.empty[st_h]);
+            umma_commit<CG>(&tl.empty[st_l]);
         }
         umma_commit<CG>(&tl.tfull[acc]);
         if (++acc == 2) {
@@ -580,19 +732,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
     const int ew = warp - 2;                  // epilogue warp 0 .. EPI_WARPS - 1
     const int quarter = warp & 3;             // TMEM lanes this warp may access
     const int half = ew >> 2;                 // column half of the tile this warp owns
-    uint32_t *T = (uint32_t *)(epi_T + (warp >= 2 ? ew : 0) * EPI_T_FLOATS);   // packed split operands
+    uint32_t *T = (uint32_t *)(epi_T + (ew >= 0 && ew < EPI_WARPS ? ew : 0) * EPI_T_FLOATS);   // packed split operands
     uint16_t *Bh = (uint16_t *)T, *Bl = Bh + EPI_BOX_ROWS * EPI_BOX_COLS;      // or the hi and lo boxes
     bool flow_first = true;                   // dataflow: no tile completed by this CTA yet
     // Epilogue: the next layer from tile w's accumulator, its FP64 partials and, in
     // the dataflow schedule, the tile's completion flag.
     auto epilogue_tile = [&](const TileWork &w) {
-        const InstDesc &d = p.inst[w.inst];
+        const InstDesc &d = rc.inst[w.inst];
         const int np = d.np;
         const size_t mat = (size_t)np * np;
-        int ok = 1;
-        if (lane == 0) ok = mbar_wait(&tl.tfull[acc], acc_phase, abort, p.timeout_ns, p.err) ? 1 : 0;
-        ok = __shfl_sync(0xffffffffu, ok, 0);
-        tc_fence_after();
         const float *__restrict__ old;
         float *__restrict__ outf;
         uint16_t *__restrict__ o1;   // hi
@@ -633,25 +781,34 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
         // ||Y||_F^2 of the next operands equals ||X||_F^2 off the diagonal (y = x
         // there); the diagonal difference y^2 - x^2 is accumulated apart (exact squares).
         FF ft = {0.f, 0.f}, fq = {0.f, 0.f}, fp = {0.f, 0.f}, fw = {0.f, 0.f};
-        if (ok && rw0 < np) {
-            // The chunks this warp finishes form one range [j0, j1): chunks entirely
-            // below the diagonal come first, chunks past np last.
-            int j0 = 0, j1 = 128 / EPI_CHUNK;
-            while (j1 > 0 && w.bj * TC_BN + half * 128 + (j1 - 1) * EPI_CHUNK >= np) --j1;
-            while (j0 < j1 && w.bj * TC_BN + half * 128 + j0 * EPI_CHUNK + EPI_CHUNK - 1 < rw0) ++j0;
-            // The previous layer's (r, c) values -- (c, r) by symmetry, coalesced across
-            // the warp, evict-first -- are loaded one chunk ahead, so that their latency
-            // overlaps the current chunk's arithmetic and stores.
-            float xnx[EPI_CHUNK];
-            if (j0 < j1) {
-                const int cb0 = w.bj * TC_BN + half * 128 + j0 * EPI_CHUNK;
+        // With narrow tiles a pass of its own (flow_record) does the sums.
+        constexpr bool NARROW = BN < 256;
+        const bool stats = !w.resp && !NARROW;
+        // The chunks this warp finishes form one range [j0, j1): chunks entirely
+        // below the diagonal come first, chunks past np last.
+        const int col0 = w.bj * BN + half * (BN / 2);   // this warp's first column
+        int j0 = 0, j1 = (rw0 < np) ? BN / 2 / EPI_CHUNK : 0;
+        while (j1 > 0 && col0 + (j1 - 1) * EPI_CHUNK >= np) --j1;
+        while (j0 < j1 && col0 + j0 * EPI_CHUNK + EPI_CHUNK - 1 < rw0) ++j0;
+        // The previous layer's (r, c) values -- (c, r) by symmetry, coalesced across
+        // the warp, evict-first -- are loaded one chunk ahead, so that their latency
+        // overlaps the current chunk's arithmetic and stores (the first chunk's, the
+        // wait for the products).
+        float xnx[EPI_CHUNK];
+        if (j0 < j1) {
+            const int cb0 = col0 + j0 * EPI_CHUNK;
 #pragma unroll
-                for (int jj = 0; jj < EPI_CHUNK; ++jj) xnx[jj] = __ldcs(old + (size_t)(cb0 + jj) * np + r);
-            }
+            for (int jj = 0; jj < EPI_CHUNK; ++jj) xnx[jj] = __ldcs(old + (size_t)(cb0 + jj) * np + r);
+        }
+        int ok = 1;
+        if (lane == 0) ok = mbar_wait(&tl.tfull[acc], acc_phase, abort, p.timeout_ns, p.err) ? 1 : 0;
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+        tc_fence_after();
+        if (ok) {
 #pragma unroll 1
             for (int j = j0; j < j1; ++j) {
-                const int c0 = half * 128 + j * EPI_CHUNK;   // column offset in the tile
-                const int cb = w.bj * TC_BN + c0;
+                const int c0 = half * (BN / 2) + j * EPI_CHUNK;   // column offset in the tile
+                const int cb = w.bj * BN + c0;
                 float xov[EPI_CHUNK];
 #pragma unroll
                 for (int jj = 0; jj < EPI_CHUNK; ++jj) xov[jj] = xnx[jj];
@@ -661,108 +818,150 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
                         xnx[jj] = __ldcs(old + (size_t)(cb + EPI_CHUNK + jj) * np + r);
                 }
                 float v[EPI_CHUNK];
-                tmem_ld16(tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * TC_BN + c0, v);
+                tmem_ld16(tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * BN + c0, v);
                 // Each element's next split operands are computed once, stored to the
                 // mirror (c, r) and staged packed (hi | lo << 16) for the direct (r, c)
                 // stores below.  The FP32 master gets the mirror and the diagonal only.
                 const bool upper = (cb > rw0 + 31);     // every element has r < c
-                // Strictly upper chunks of plain layers write their direct (r, c) operands
-                // as two boxes of tensor stores; the others through the transpose buffer,
-                // once the previous chunk's boxes have left it.
-                const bool boxed = upper && !accel;
-                if (!boxed) {
+                // Strictly upper chunks write their direct (r, c) operands as two boxes of
+                // tensor stores; the diagonal ones through the transpose buffer, once the
+                // previous chunk's boxes have left it.
+                if (!upper) {
                     if (lane == 0) bulk_wait_read();
                     __syncwarp();
                 }
                 uint32_t hp[EPI_CHUNK / 2], lp[EPI_CHUNK / 2];   // (r, c), (r, c + 1) packed
-                if (upper && !w.resp && !accel) {
-                    // The common case: a plain square-chain layer, strictly upper chunk.
-                    const float twoc = 2.0f * cf;
+                float x[EPI_CHUNK];
+                if (upper) {
+                    if (!w.resp && !accel) {   // a plain square
+                        const float twoc = 2.0f * cf;
 #pragma unroll
-                    for (int jj = 0; jj < EPI_CHUNK; ++jj) {
-                        const int c = cb + jj;
-                        const float xo = xov[jj];
-                        const float t = fmaf(twoc, xo, v[jj] * unscale);
-                        const float x = w.flip ? xo - t : t + xo;   // 2X - X^2 or X^2
-                        ff_add_sq(fq, x, 2.0f);
-                        const size_t m = (size_t)c * np + r;
-                        __stcs(outf + m, x);
-                        uint16_t a1, a2;
-                        split2<PREC, X_SHIFT>(x, a1, a2);
-                        __stcs(o1 + m, a1);
-                        __stcs(o2 + m, a2);
-                        pack_pair(hp, lp, jj, a1, a2);
+                        for (int jj = 0; jj < EPI_CHUNK; ++jj) {
+                            const float xo = xov[jj];
+                            const float t = fmaf(twoc, xo, v[jj] * unscale);
+                            x[jj] = w.flip ? xo - t : t + xo;   // 2X - X^2 or X^2
+                        }
+                    } else if (!w.resp) {
+                        const float twoc = 2.0f * cf;
+#pragma unroll
+                        for (int jj = 0; jj < EPI_CHUNK; ++jj)
+                            x[jj] = fmaf(ka, fmaf(twoc, xov[jj], v[jj] * unscale), kb * xov[jj]);
+                    } else if (!accel) {
+                        // Response / adjoint stream: P = Y X1 + X1 Y; with X = Y + (1/2 + c) I
+                        // the chain needs X X1 + X1 X = P + (1 + 2c) X1, negated for 2X - X^2.
+                        const float kx = w.flip ? 1.0f - 2.0f * cf : 1.0f + 2.0f * cf;
+                        const float sg = w.flip ? -unscale : unscale;
+#pragma unroll
+                        for (int jj = 0; jj < EPI_CHUNK; ++jj) x[jj] = fmaf(kx, xov[jj], v[jj] * sg);
+                    } else {
+#pragma unroll
+                        for (int jj = 0; jj < EPI_CHUNK; ++jj) x[jj] = fmaf(kx1, xov[jj], ka * (v[jj] * unscale));
                     }
-                } else if (upper && w.resp && !accel) {
-                    // Response / adjoint stream, plain layer, strictly upper chunk:
-                    // X X1 + X1 X = P + (1 + 2c) X1, negated for 2X - X^2 (as below).
-                    const float kx = w.flip ? 1.0f - 2.0f * cf : 1.0f + 2.0f * cf;
-                    const float sg = w.flip ? -unscale : unscale;
+                    if (stats) {
+#pragma unroll
+                        for (int jj = 0; jj < EPI_CHUNK; ++jj) ff_add_sq(fq, x[jj], 2.0f);
+                    }
+                    // Mirror (c, r): the FP32 master one column per store; the operands two
+                    // rows packed per lane, exchanged with the neighbour so that the even
+                    // lane stores rows (r, r + 1) of column c and the odd one rows
+                    // (r - 1, r) of column c + 1.
+                    float *mf = outf + (size_t)cb * np + r;
 #pragma unroll
                     for (int jj = 0; jj < EPI_CHUNK; ++jj) {
-                        const int c = cb + jj;
-                        const float x = fmaf(kx, xov[jj], v[jj] * sg);
-                        const size_t m = (size_t)c * np + r;
-                        __stcs(outf + m, x);
-                        uint16_t a1, a2;
-                        split2<PREC, Y_SHIFT>(x, a1, a2);
-                        __stcs(o1 + m, a1);
-                        __stcs(o2 + m, a2);
-                        pack_pair(hp, lp, jj, a1, a2);
+                        __stcs(mf, x[jj]);   // streaming stores: keep L2 for the operands
+                        mf += np;
+                    }
+                    const int odd = lane & 1;
+                    const uint32_t sel = odd ? 0x3276u : 0x5410u;
+                    size_t m = (size_t)(cb + odd) * np + (r - odd);
+#pragma unroll
+                    for (int k = 0; k < EPI_CHUNK / 2; ++k) {
+                        if (!w.resp) split2_pair<PREC, X_SHIFT>(x[2 * k], x[2 * k + 1], hp[k], lp[k]);
+                        else split2_pair<PREC, Y_SHIFT>(x[2 * k], x[2 * k + 1], hp[k], lp[k]);
+                        const uint32_t hn = __shfl_xor_sync(0xffffffffu, hp[k], 1);
+                        const uint32_t ln = __shfl_xor_sync(0xffffffffu, lp[k], 1);
+                        __stcs((uint32_t *)(o1 + m), __byte_perm(hp[k], hn, sel));
+                        __stcs((uint32_t *)(o2 + m), __byte_perm(lp[k], ln, sel));
+                        m += 2 * (size_t)np;
                     }
                 } else {
+                    // A chunk on the diagonal: selects instead of branches, and the lane's
+                    // diagonal element (at most one, column jd) apart.
+                    const int jd = r - cb;
+                    const bool dreal = r < nreal;
+                    if (!w.resp) {
+                        // P = Y^2 for the stored operands Y = X - I/2; the true input is
+                        // X + cI, so X^2 = P + 2cY + cI + X - I/4 (c^2 is below FP32 here).
+                        const float twoc = 2.0f * cf;
+                        const float cd = dreal ? (w.flip ? -cf : cf) : 0.0f, qd = dreal ? 0.25f : 0.0f;
+                        const float hd = dreal ? 0.5f : 0.0f, kcd = dreal ? kc : 0.0f, cfd = dreal ? cf : 0.0f;
 #pragma unroll
-                    for (int jj = 0; jj < EPI_CHUNK; ++jj) {
-                        const int c = cb + jj;
-                        const float P = v[jj] * unscale;            // raw product
-                        const float xo = xov[jj];
-                        const bool dg = (r == c) && (r < nreal);
-                        float x;
-                        if (!w.resp) {
-                            // P = Y^2 for the stored operands Y = X - I/2; the true input is
-                            // X + cI, so X^2 = P + 2cY + cI + X - I/4 (c^2 is below FP32 here).
-                            const float yo = dg ? xo - 0.5f : xo;
+                        for (int jj = 0; jj < EPI_CHUNK; ++jj) {
+                            const bool dg = jj == jd;
+                            const float P = v[jj] * unscale;            // raw product
+                            const float xo = xov[jj];
+                            const float yo = dg ? xo - hd : xo;
                             if (accel) {
-                                x = fmaf(ka, fmaf(2.0f * cf, yo, P), fmaf(kb, dg ? yo + cf : yo, dg ? kc : 0.0f));
+                                x[jj] = fmaf(ka, fmaf(twoc, yo, P), fmaf(kb, dg ? yo + cfd : yo, dg ? kcd : 0.0f));
                             } else {
-                                const float b = dg ? P - 0.25f : P;
-                                if (!w.flip) x = (b + fmaf(2.0f * cf, yo, dg ? cf : 0.0f)) + xo;  // X^2
-                                else x = xo - (b + fmaf(2.0f * cf, yo, dg ? -cf : 0.0f));        // 2X - X^2
-                            }
-                        } else if (accel) {
-                            x = fmaf(kx1, xo, ka * P);
-                        } else {
-                            // P = Y X1 + X1 Y; with X = Y + (1/2 + c) I the chain needs
-                            // X X1 + X1 X = P + (1 + 2c) X1.
-                            x = w.flip ? fmaf(1.0f - 2.0f * cf, xo, -P) : fmaf(1.0f + 2.0f * cf, xo, P);
-                        }
-                        const float y = (dg && !w.resp) ? x - 0.5f : x;  // next operands
-                        uint16_t a1, a2;
-                        if (!w.resp) split2<PREC, X_SHIFT>(y, a1, a2);
-                        else split2<PREC, Y_SHIFT>(y, a1, a2);
-                        if (r <= c) {
-                            if (!w.resp) {
-                                ff_add_sq(fq, x, (r == c) ? 1.0f : 2.0f);
-                                if (r == c) ff_add(ft, x);
-                                if (dg) {
-                                    ff_add(fp, P);
-                                    ff_add_sq(fw, y, 1.0f);
-                                    ff_add_sq(fw, x, -1.0f);
-                                }
-                            }
-                            // mirror (c, r), consecutive r across the warp; the diagonal
-                            // element's FP32 master value here too
-                            const size_t m = (size_t)c * np + r;
-                            __stcs(outf + m, x);   // streaming stores: keep L2 for the operands
-                            if (r < c) {
-                                __stcs(o1 + m, a1);
-                                __stcs(o2 + m, a2);
+                                const float t = (dg ? P - qd : P) + fmaf(twoc, yo, dg ? cd : 0.0f);
+                                x[jj] = w.flip ? xo - t : t + xo;   // 2X - X^2 or X^2
                             }
                         }
-                        T[lane * (EPI_CHUNK + 1) + jj] = (uint32_t)a1 | ((uint32_t)a2 << 16);
+                    } else {
+                        const float kx = accel ? kx1 : w.flip ? 1.0f - 2.0f * cf : 1.0f + 2.0f * cf;
+                        const float sg = accel ? ka : w.flip ? -1.0f : 1.0f;
+#pragma unroll
+                        for (int jj = 0; jj < EPI_CHUNK; ++jj) x[jj] = fmaf(kx, xov[jj], sg * (v[jj] * unscale));
+                    }
+                    if (!w.resp) {
+                        float xd = 0.0f, Pd = 0.0f;
+#pragma unroll
+                        for (int jj = 0; jj < EPI_CHUNK; ++jj) {
+                            if (!NARROW) ff_add_sq(fq, jj >= jd ? x[jj] : 0.0f, jj == jd ? 1.0f : 2.0f);
+                            if (jj == jd) {
+                                xd = x[jj];
+                                Pd = v[jj] * unscale;
+                            }
+                        }
+                        if (NARROW) {
+                            if (jd >= 0 && jd < EPI_CHUNK) __stcg(d.pdiag[(w.n + 1) & 1] + r, Pd);
+                        } else if (jd >= 0 && jd < EPI_CHUNK) {
+                            ff_add(ft, xd);
+                            if (dreal) {
+                                ff_add(fp, Pd);
+                                ff_add_sq(fw, xd - 0.5f, 1.0f);
+                                ff_add_sq(fw, xd, -1.0f);
+                            }
+                        }
+                    }
+                    // mirror (c, r), consecutive r across the warp, and the diagonal of the
+                    // FP32 master: streaming stores, keep L2 for the operands
+                    size_t m = (size_t)cb * np + r;
+#pragma unroll
+                    for (int k = 0; k < EPI_CHUNK / 2; ++k) {
+                        const int j0k = 2 * k, j1k = 2 * k + 1;
+                        const float h = (dreal && !w.resp) ? 0.5f : 0.0f;   // next operands: Y = X - I/2
+                        const float y0 = j0k == jd ? x[j0k] - h : x[j0k], y1 = j1k == jd ? x[j1k] - h : x[j1k];
+                        if (!w.resp) split2_pair<PREC, X_SHIFT>(y0, y1, hp[k], lp[k]);
+                        else split2_pair<PREC, Y_SHIFT>(y0, y1, hp[k], lp[k]);
+                        if (j0k >= jd) __stcs(outf + m, x[j0k]);
+                        if (j0k > jd) {
+                            __stcs(o1 + m, (uint16_t)hp[k]);
+                            __stcs(o2 + m, (uint16_t)lp[k]);
+                        }
+                        m += np;
+                        if (j1k >= jd) __stcs(outf + m, x[j1k]);
+                        if (j1k > jd) {
+                            __stcs(o1 + m, (uint16_t)(hp[k] >> 16));
+                            __stcs(o2 + m, (uint16_t)(lp[k] >> 16));
+                        }
+                        m += np;
+                        T[lane * (EPI_CHUNK + 1) + j0k] = __byte_perm(hp[k], lp[k], 0x5410);
+                        T[lane * (EPI_CHUNK + 1) + j1k] = __byte_perm(hp[k], lp[k], 0x7632);
                     }
                 }
-                if (boxed) {
+                if (upper) {
                     // The chunk's 32 x 16 boxes of hi and lo, row-major, to global memory
                     // by the tensor store unit (the operands need both triangles: TMA
                     // loads rows).
@@ -782,18 +981,21 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
                     }
                 } else {
                     __syncwarp();
-                    // direct (r, c) split-operand stores through the transpose buffer, two
-                    // rows per step: lanes 0..15 row ii, lanes 16..31 row ii + 1
-                    const int hl = lane >> 4, cl = lane & 15;
-#pragma unroll 4
-                    for (int it = 0; it < 16; ++it) {
-                        const int ii = 2 * it + hl;
+                    // direct (r, c) split-operand stores through the transpose buffer: eight
+                    // lanes a row, two columns each, on and above the diagonal
+                    const int hl = lane >> 3, cl = 2 * (lane & 7);
+#pragma unroll
+                    for (int it = 0; it < 8; ++it) {
+                        const int ii = 4 * it + hl;
                         const int rr = rw0 + ii, cc = cb + cl;
-                        if (upper || rr <= cc) {
-                            const uint32_t pk = T[ii * (EPI_CHUNK + 1) + cl];
-                            const size_t m = (size_t)rr * np + cc;
-                            __stcs(o1 + m, (uint16_t)(pk & 0xFFFFu));
-                            __stcs(o2 + m, (uint16_t)(pk >> 16));
+                        const uint32_t u0 = T[ii * (EPI_CHUNK + 1) + cl], u1 = T[ii * (EPI_CHUNK + 1) + cl + 1];
+                        const size_t md = (size_t)rr * np + cc;
+                        if (rr <= cc) {
+                            __stcs((uint32_t *)(o1 + md), __byte_perm(u0, u1, 0x5410));
+                            __stcs((uint32_t *)(o2 + md), __byte_perm(u0, u1, 0x7632));
+                        } else if (rr == cc + 1) {
+                            __stcs(o1 + md + 1, (uint16_t)u1);
+                            __stcs(o2 + md + 1, (uint16_t)(u1 >> 16));
                         }
                     }
                     __syncwarp();
@@ -812,76 +1014,129 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
             acc = 0;
             acc_phase ^= 1u;
         }
-        if (!w.resp) {
-            // The tile's partials stay compensated FP32 pairs through the warp and
-            // cross-warp sums (FP64 arithmetic is slow on this part); one conversion.
-            FF qw = fq;
-            ff_add_ff(qw, fw);
-            const FF r4[4] = {ff_warp_sum(ft), ff_warp_sum(fq), ff_warp_sum(qw), ff_warp_sum(fp)};
-            if (lane == 0)
-#pragma unroll
-                for (int k = 0; k < 4; ++k) tl.red[ew][k] = r4[k];
-            if (p.dataflow) {
-                // This warp's stores (generic proxy, and its tensor stores once
-                // complete) reach the TMA reads (async proxy) of any CTA that sees the
-                // tile's completion flag (the flag's writer fences for the CTA after
-                // the barrier below).
-                if (lane == 0) {
-                    bulk_wait_all();
-                    __threadfence();
-                }
+        if (stats) {
+            write_record(tl.red, d.part[(w.n + 1) % 3] + w.tile * CG + (int)rank, ft, fq, fw, fp, ew, lane);
+            asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32) : "memory");   // the buffer is free again
+        }
+        if (SCHED != RUN_ROUNDS) {
+            // This warp's stores (generic proxy, and its tensor stores once complete)
+            // reach the TMA reads (async proxy) of any CTA that sees its completion.
+            asm volatile("fence.proxy.async.global;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) {
+                bulk_wait_all();
                 asm volatile("fence.proxy.async.global;" ::: "memory");
-            }
-            asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32) : "memory");
-            if (ew == 0 && lane == 0) {
-                FF a4[4] = {tl.red[0][0], tl.red[0][1], tl.red[0][2], tl.red[0][3]};
-                for (int k = 1; k < EPI_WARPS; ++k)
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) ff_add_ff(a4[c], tl.red[k][c]);
-                Part s4;
-                s4.t = ff_value(a4[0]);
-                s4.q = ff_value(a4[1]);
-                s4.w = ff_value(a4[2]);
-                s4.p = ff_value(a4[3]);
-                d.part[(w.n + 1) % 3][w.tile * CG + (int)rank] = s4;
-                if (p.dataflow) {
-                    __threadfence();
-                    // test_hook: CTA 0 withholds its first completion (a CTA that never
-                    // finishes; the other CTAs' waits must run out).
-                    if (!(p.test_hook == 1 && blockIdx.x == 0 && w.n == 0 && flow_first)) {
+                __threadfence();
+                // test_hook: CTA 0's first epilogue warp withholds its first completion (a
+                // CTA that never finishes; the other CTAs' waits must run out).
+                if (!(p.test_hook == 1 && blockIdx.x == 0 && ew == 0 && w.n == 0 && flow_first)) {
+                    if (SCHED == RUN_BATCH) {
+                        atomicAdd(&d.ctl->flow_done, 1u);
+                    } else {
                         atomicAdd(p.tile_done + w.tile, 1u);
                         atomicAdd(p.layer_done, 1u);
                     }
-                    flow_first = false;
                 }
             }
-            if (p.publish && ew == 0) {
-                // Round schedule of a density batch: the CTA whose record completes the
-                // instance's layer sums it (the order of every CTA's own sum) and
-                // publishes the sums for the decision after the grid barrier.
-                int last = 0;
-                if (lane == 0) {
-                    __threadfence();
-                    const unsigned int target = (unsigned int)(w.n + 1) * (unsigned int)d.parts;
-                    last = (atomicAdd(&d.ctl->psum_done, 1u) + 1u == target) ? 1 : 0;
-                }
-                last = __shfl_sync(0xffffffffu, last, 0);
-                if (last) {
-                    __threadfence();   // the other CTAs' records, released before their increments
-                    double a[4];
-                    sum_layer_partials(p, w.inst, w.n + 1, lane, a);
-                    if (lane == 0) {
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) d.ctl->psum[c] = a[c];
-                        d.ctl->psum_n = w.n + 1;
-                    }
-                }
-            }
-            asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32) : "memory");
+            flow_first = false;
         }
     };
 
-    if (p.dataflow) {
+    // A list of `total` tiles (largest instances first) is dealt to the pairs in a snake
+    // order, forward in even waves and backward in odd ones, which evens out the pairs'
+    // shares of large and small tiles; each pair then takes its share smallest first, so
+    // that the epilogues of its small tiles overlap the MMAs of the large ones after them.
+    const auto round_tile = [&](int k) {
+        return k * nclusters + ((k & 1) ? nclusters - 1 - cluster_id : cluster_id);
+    };
+    const auto round_count = [&](int total) {
+        int nk = 0;
+        while (round_tile(nk) < total) ++nk;
+        return nk;
+    };
+
+    if constexpr (SCHED == RUN_BATCH) {
+        // ------------------ dataflow schedule of a batch (density mode) ------------------
+        const int nk = round_count(rc.prefix[p.B]);
+        const auto tile_of = [&](int g, int r) {
+            TileWork w;
+            map_tile(rc, p.B, rc.inst, g, w.inst, w.job, w.tile);
+            const TileWork f = describe_flow(rc, w.tile, p.tiles[rc.inst[w.inst].tile_off + w.tile], r);
+            w.bi = f.bi;
+            w.bj = f.bj;
+            w.resp = w.ybuf = w.flip = w.rec = 0;
+            w.xslot = xslot_of(rc.inst[w.inst], r);
+            w.n = r;
+            w.cf = 0.0f;
+            w.alpha = 1.0f;
+            return w;
+        };
+        bool any = nk > 0;
+        if (warp == 0) {
+            if (lane == 0)
+                for (int r = 0; any && !*abort; ++r) {
+                    any = false;
+                    for (int k = nk - 1; k >= 0 && !*abort; --k) {
+                        const TileWork w = tile_of(round_tile(k), r);
+                        const int go = flow_wait_instance(p, rc.inst[w.inst].ctl, r, abort);
+                        if (go < 0) tc_abort<CG>(rc, peer_abort);
+                        if (go <= 0) continue;
+                        any = true;
+                        asm volatile("fence.proxy.async.global;" ::: "memory");
+                        produce_tile(w);
+                    }
+                }
+        } else if (warp == 1) {
+            if (leader)
+                for (int r = 0; any; ++r) {
+                    any = false;
+                    for (int k = nk - 1; k >= 0; --k) {
+                        const TileWork w = tile_of(round_tile(k), r);
+                        int go = 0;
+                        if (lane == 0) go = flow_wait_instance(p, rc.inst[w.inst].ctl, r, abort);
+                        go = __shfl_sync(0xffffffffu, go, 0);
+                        if (go < 0) tc_abort<CG>(rc, peer_abort);
+                        if (go > 0) {
+                            any = true;
+                            if (!mma_tile(w)) go = -1;
+                        }
+                        if (go < 0) {
+                            any = false;
+                            break;
+                        }
+                    }
+                }
+        } else if (warp < 2 + EPI_WARPS) {
+            for (int r = 0; any; ++r) {
+                any = false;
+                for (int k = nk - 1; k >= 0; --k) {
+                    TileWork w = tile_of(round_tile(k), r);
+                    const InstCtl *ctl = rc.inst[w.inst].ctl;
+                    int go = 0;
+                    if (lane == 0) {
+                        go = flow_wait_instance(p, ctl, r, abort);
+                        w.flip = __ldcg(&ctl->flow_flip);
+                        w.cf = __ldcg(&ctl->flow_cf);
+                        w.alpha = __ldcg(&ctl->flow_alpha);
+                    }
+                    go = __shfl_sync(0xffffffffu, go, 0);
+                    if (go < 0) {
+                        tc_abort<CG>(rc, peer_abort);
+                        any = false;
+                        break;
+                    }
+                    if (go == 0) continue;
+                    any = true;
+                    w.flip = __shfl_sync(0xffffffffu, w.flip, 0);
+                    w.cf = __shfl_sync(0xffffffffu, w.cf, 0);
+                    w.alpha = __shfl_sync(0xffffffffu, w.alpha, 0);
+                    epilogue_tile(w);
+                }
+            }
+        } else {
+            flow_owner<CG>(rc, p, lane, abort);
+        }
+    } else if constexpr (SCHED == RUN_FLOW) {
         // ------------- dataflow schedule (one instance, density mode) -------------
         // No grid barrier between layers.  The producer and the MMA thread run on into
         // the next layer as soon as their own tiles are done (the producer waits per
@@ -891,7 +1146,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
         // rule fires they halt the CTA: loads and MMAs issued ahead are drained at
         // teardown.  Each tile's arithmetic, and so X and D, is that of the barrier
         // schedule bit for bit.
-        const int ntl = p.inst[0].ntiles;
+        const int ntl = rc.inst[0].ntiles;
+        const int2 *tiles = p.tiles + rc.inst[0].tile_off;
         // When every pair has a few tiles in every layer (fewer than four), layer r's
         // round-robin starts at a rotated position, so that the pairs holding one
         // tile fewer change from layer to layer and the remainder tiles spread evenly
@@ -907,21 +1163,31 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
         } else if (warp == 0) {
             if (lane == 0)
                 for (int r = 0; !*abort; ++r)
-                    for (int g = first_tile(r); g < ntl && !*abort; g += nclusters) produce_tile(describe_flow(p, g, r));
+                    for (int g = first_tile(r); g < ntl && !*abort; g += nclusters) produce_tile(describe_flow(rc, g, tiles[g], r));
         } else if (warp == 1) {
-            if (lane == 0 && leader) {
+            if (leader) {
                 bool ok = true;
-                for (int r = 0; ok && !*abort; ++r)
-                    for (int g = first_tile(r); ok && g < ntl && !*abort; g += nclusters)
-                        ok = mma_tile(describe_flow(p, g, r));
+                for (int r = 0; ok; ++r)
+                    for (int g = first_tile(r); ok && g < ntl; g += nclusters)
+                        ok = mma_tile(describe_flow(rc, g, tiles[g], r));
             }
-        } else {
+        } else if (warp < 2 + EPI_WARPS) {
             for (int r = 0;; ++r) {
-                if (!flow_decide(rc, p, tl.flow_sums, r, ew, lane, ntl * CG, abort)) {
+                const int g0 = first_tile(r);
+                int2 bt = make_int2(0, 0);
+                if (g0 < ntl) bt = tiles[g0];   // ahead of the wait
+                if (!flow_decide<(BN < 256)>(rc, tl.red, tl.flow_sums, p, r, ew, lane, (unsigned int)(EPI_WARPS * CG * ntl), abort)) {
                     tc_abort<CG>(rc, peer_abort);   // stop rule or error: halt this CTA and its peer
                     break;
                 }
-                for (int g = first_tile(r); g < rc.total; g += nclusters) epilogue_tile(describe(rc, p, g));
+                for (int g = g0; g < ntl; g += nclusters) {
+                    if (g != g0) bt = tiles[g];
+                    TileWork w = describe_flow(rc, g, bt, r);
+                    w.flip = rc.choice[0] == SP2_CHOICE_FLIP;
+                    w.cf = (float)rc.coff[0];
+                    w.alpha = rc.alpha[0];
+                    epilogue_tile(w);
+                }
             }
         }
     } else {
@@ -955,24 +1221,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
             __syncthreads();
             if (rc.abort || rc.total == 0) break;
 
-            // The round's tiles (largest instances first) are dealt to the pairs in a
-            // snake order, forward in even waves and backward in odd ones, which evens
-            // out the pairs' shares of large and small tiles; each pair then takes its
-            // share smallest first, so that the epilogues of its small tiles overlap
-            // the MMAs of the large ones after them.
-            const auto round_tile = [&](int k) {
-                return k * nclusters + ((k & 1) ? nclusters - 1 - cluster_id : cluster_id);
-            };
-            int nk = 0;
-            while (round_tile(nk) < rc.total) ++nk;
+            const int nk = round_count(rc.total);
             if (warp == 0) {
                 if (lane == 0)
                     for (int k = nk - 1; k >= 0 && !*abort; --k) produce_tile(describe(rc, p, round_tile(k)));
             } else if (warp == 1) {
-                if (lane == 0 && leader)
-                    for (int k = nk - 1; k >= 0 && !*abort; --k)
+                if (leader)
+                    for (int k = nk - 1; k >= 0; --k)
                         if (!mma_tile(describe(rc, p, round_tile(k)))) break;
-            } else {
+            } else if (warp < 2 + EPI_WARPS) {
                 for (int k = nk - 1; k >= 0; --k) epilogue_tile(describe(rc, p, round_tile(k)));
                 // This warp's tensor stores are complete; order this round's
                 // generic-proxy stores before the async-proxy (TMA) reads of the next
@@ -987,10 +1244,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
 
     // ------------------------------ teardown ------------------------------
     // Tensor stores still reading this CTA's shared memory finish before it is released.
-    if (warp >= 2 && lane == 0) bulk_wait_all();
+    if (warp >= 2 && warp < 2 + EPI_WARPS && lane == 0) bulk_wait_all();
     // After an abort: MMAs this launch issued complete before tensor memory and the
     // stages are released (the commit covers every earlier MMA of the issuing thread).
-    if (warp == 1 && lane == 0 && leader && rc.abort) {
+    if (warp == 1 && leader && __any_sync(0xffffffffu, *abort)) {
         umma_commit<CG>(&tl.drain);
         const unsigned long long t0 = global_ns();
         while (!mbar_try_wait(&tl.drain, 0u) && global_ns() - t0 < p.timeout_ns) {
@@ -1040,38 +1297,50 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
     if (warp == 1) {
         tc_fence_after();
         if (CG == 2)
-            asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS)
+            asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(C::TMEM_COLS)
                          : "memory");
         else
-            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS)
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(C::TMEM_COLS)
                          : "memory");
     }
 }
 
-template <int CG>
-const void *tc_kernel_ptr(int precision) {
-    return (precision == SP2_BF16_SPLIT) ? (const void *)k_tc_persistent<SP2_BF16_SPLIT, CG>
-                                         : (const void *)k_tc_persistent<SP2_FP16_SPLIT, CG>;
+template <int CG, int BN, int SCHED>
+const void *tc_kernel_of(int precision) {
+    return (precision == SP2_BF16_SPLIT) ? (const void *)k_tc_persistent<SP2_BF16_SPLIT, CG, BN, SCHED>
+                                         : (const void *)k_tc_persistent<SP2_FP16_SPLIT, CG, BN, SCHED>;
+}
+// The tile shapes: 256 x 256 and 128 x 256 with every schedule, 256 x 128 and 128 x 64
+// for a lone density solve.
+const void *tc_kernel_ptr(int precision, int cg, int bn, int sched) {
+    if (sched == RUN_BATCH)
+        return cg == 2 ? tc_kernel_of<2, 256, RUN_BATCH>(precision) : tc_kernel_of<1, 256, RUN_BATCH>(precision);
+    if (sched == RUN_ROUNDS)
+        return cg == 2 ? tc_kernel_of<2, 256, RUN_ROUNDS>(precision) : tc_kernel_of<1, 256, RUN_ROUNDS>(precision);
+    if (cg == 2) return bn == 128 ? tc_kernel_of<2, 128, RUN_FLOW>(precision) : tc_kernel_of<2, 256, RUN_FLOW>(precision);
+    return bn == 64 ? tc_kernel_of<1, 64, RUN_FLOW>(precision) : tc_kernel_of<1, 256, RUN_FLOW>(precision);
 }
 
 }  // namespace
 
 static_assert(SMEM_BYTES <= 232448, "dynamic shared memory above the 227 KB a CTA can hold");
-size_t tc_smem_bytes() { return SMEM_BYTES; }
 
-// Number of CTAs of a co-resident persistent grid for the given CTA group size
+// Number of CTAs of a co-resident persistent grid for the given tile shape
 // (0 when the configuration cannot be launched on this device).
-int tc_grid_size(int cta_group, int sm_count) {
-    const void *fns[2] = {cta_group == 2 ? tc_kernel_ptr<2>(SP2_FP16_SPLIT) : tc_kernel_ptr<1>(SP2_FP16_SPLIT),
-                          cta_group == 2 ? tc_kernel_ptr<2>(SP2_BF16_SPLIT) : tc_kernel_ptr<1>(SP2_BF16_SPLIT)};
-    for (const void *f : fns)
-        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES) != cudaSuccess) {
-            cudaGetLastError();
-            return 0;
+int tc_grid_size(int cta_group, int bn, int sm_count) {
+    const void *fn = nullptr;
+    for (int prec : {SP2_FP16_SPLIT, SP2_BF16_SPLIT})
+        for (int sched : {RUN_ROUNDS, RUN_FLOW, RUN_BATCH}) {
+            fn = tc_kernel_ptr(prec, cta_group, bn, sched);
+            if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES) != cudaSuccess) {
+                cudaGetLastError();
+                return 0;
+            }
         }
+    fn = tc_kernel_ptr(SP2_FP16_SPLIT, cta_group, bn, RUN_FLOW);
     if (cta_group == 1) {
         int b = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fns[0], TC_THREADS, SMEM_BYTES) != cudaSuccess) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, TC_THREADS, SMEM_BYTES) != cudaSuccess) {
             cudaGetLastError();
             return 0;
         }
@@ -1089,7 +1358,7 @@ int tc_grid_size(int cta_group, int sm_count) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int nclusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&nclusters, fns[0], &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&nclusters, fn, &cfg) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -1097,7 +1366,7 @@ int tc_grid_size(int cta_group, int sm_count) {
     return nclusters * 2;
 }
 
-cudaError_t launch_tc_persistent(const RunParams &p, int cta_group, int grid, cudaStream_t s) {
+cudaError_t launch_tc_persistent(const RunParams &p, int cta_group, int bn, int grid, cudaStream_t s) {
     void *args[] = {(void *)&p};
     if (cta_group == 1) {
         // Cooperative launch (co-residency of the whole grid), through the
@@ -1112,7 +1381,7 @@ cudaError_t launch_tc_persistent(const RunParams &p, int cta_group, int grid, cu
         cfg.stream = s;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        return cudaLaunchKernelExC(&cfg, tc_kernel_ptr<1>(p.precision), args);
+        return cudaLaunchKernelExC(&cfg, tc_kernel_ptr(p.precision, 1, bn, p.dataflow), args);
     }
     // CTA pairs: a cluster launch of exactly as many pairs as the device holds
     // at once (cudaOccupancyMaxActiveClusters, one CTA per SM), so on an idle GPU
@@ -1132,7 +1401,7 @@ cudaError_t launch_tc_persistent(const RunParams &p, int cta_group, int grid, cu
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelExC(&cfg, tc_kernel_ptr<2>(p.precision), args);
+    return cudaLaunchKernelExC(&cfg, tc_kernel_ptr(p.precision, 2, bn, p.dataflow), args);
 }
 
 }  // namespace sp2i

@@ -72,28 +72,49 @@ __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wa
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// K-major operand in the 128-byte swizzle layout written by TMA: rows of 128 B,
-// 8-row atoms 1024 B apart (stride byte offset), descriptor version 1.
-__device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr) {
-    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) |
-           ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+// The MMA warp runs as a whole (its loop, waits and descriptors are warp-uniform, so
+// they live in the uniform datapath that tcgen05 takes its operands from) and one
+// elected lane, the same each time, issues.
+
+// A warp's wait, with a uniform result.  Every lane tries once, which suspends until
+// the phase completes or a time limit of the hardware, and lane 0 alone goes on from
+// there.  (Lane 0 alone from the start made a layer at N = 8192 1130 us instead of
+// 747; all lanes to the end made a stopped launch's last waits take a millisecond.)
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity, const volatile int *abort,
+                                               unsigned long long timeout_ns, int *err) {
+    int ok = 1;
+    if (!mbar_try_wait(bar, parity) && (threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity, abort, timeout_ns, err) ? 1 : 0;
+    return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 
+// K-major operand in the 128-byte swizzle layout written by TMA: rows of 128 B,
+// 8-row atoms 1024 B apart (stride byte offset), descriptor version 1.  The low word
+// holds the address / 16 (K steps of 32 B add 2), the high word is constant.
+constexpr uint32_t SDESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);
+__device__ __forceinline__ uint32_t sdesc_lo(uint32_t saddr) { return ((saddr & 0x3FFFFu) >> 4) | (1u << 16); }
+
 template <int CG>
-__device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+__device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc,
+                                         uint32_t accumulate) {
     if (CG == 2)
         asm volatile(
-            "{\n\t.reg .pred p;\n\t"
+            "{\n\t.reg .pred p, e;\n\t.reg .b64 a, b;\n\t"
+            "elect.sync _|e, 0xffffffff;\n\t"
             "setp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-            "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
+            "mov.b64 a, {%1, %5};\n\t"
+            "mov.b64 b, {%2, %5};\n\t"
+            "@e tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %3, p;\n\t}\n" ::"r"(d_tmem),
+            "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(accumulate), "r"(SDESC_HI)
             : "memory");
     else
         asm volatile(
-            "{\n\t.reg .pred p;\n\t"
+            "{\n\t.reg .pred p, e;\n\t.reg .b64 a, b;\n\t"
+            "elect.sync _|e, 0xffffffff;\n\t"
             "setp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
-            "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
+            "mov.b64 a, {%1, %5};\n\t"
+            "mov.b64 b, {%2, %5};\n\t"
+            "@e tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n\t}\n" ::"r"(d_tmem),
+            "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(accumulate), "r"(SDESC_HI)
             : "memory");
 }
 // Arrive on `bar` once the MMAs issued so far have completed; for a CTA pair the
@@ -103,13 +124,19 @@ __device__ __forceinline__ void umma_commit(uint64_t *bar) {
     if (CG == 2) {
         const uint16_t both = 3;
         asm volatile(
-            "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-                smem_u32(bar)),
+            "{\n\t.reg .pred e;\n\t"
+            "elect.sync _|e, 0xffffffff;\n\t"
+            "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], "
+            "%1;\n\t}\n" ::"r"(smem_u32(bar)),
             "h"(both)
             : "memory");
     } else {
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                     : "memory");
+        asm volatile(
+            "{\n\t.reg .pred e;\n\t"
+            "elect.sync _|e, 0xffffffff;\n\t"
+            "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n" ::"r"(
+                smem_u32(bar))
+            : "memory");
     }
 }
 
