@@ -23,7 +23,7 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libsp2.so")
 SOURCES = ["aux_kernels.cu", "simt_kernel.cu", "tc_kernel.cu", "exact_kernel.cu", "api.cu", "noalloc.cu",
-           "fp64_ext.cu", "host_link.cu"]
+           "fp64_ext.cu", "host_link.cu", "device_pool.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", f"-I{INCLUDE}", f"-I{CSRC}"]
 

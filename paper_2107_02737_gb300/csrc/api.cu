@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "device_common.cuh"
+#include "device_pool.h"
 #include "host_link.h"
 
 using namespace sp2i;
@@ -115,31 +116,6 @@ struct InstSpec {
     const sp2_stats *fwd = nullptr;
     const int *choices = nullptr;  // apply mode (host)
     int nchoices = -1;
-};
-
-// Device allocation owned by one call; freed on every exit path.  With `fail`
-// set (sp2_opts.test_hook = 2, host-side fault injection) every allocation
-// reports failure, as an exhausted device would.
-struct Arena {
-    std::vector<void *> ptrs;
-    cudaStream_t s;
-    bool fail = false;
-    explicit Arena(cudaStream_t st) : s(st) {}
-    void *get(size_t bytes) {
-        void *p = nullptr;
-        if (bytes == 0) bytes = 256;
-        if (fail) return nullptr;
-        if (cudaMallocAsync(&p, bytes, s) != cudaSuccess) {
-            cudaGetLastError();
-            return nullptr;
-        }
-        ptrs.push_back(p);
-        return p;
-    }
-    ~Arena() {
-        for (void *p : ptrs) cudaFreeAsync(p, s);
-        cudaStreamSynchronize(s);
-    }
 };
 
 struct Carver {
@@ -537,7 +513,7 @@ sp2_status choose_launch(Plan &pl, int want, int &grid) {
 // (the workspace tail, else `arena`) when `staging_ok`; otherwise they are an
 // argument error.
 sp2_status prepare(Prepared &P, const sp2_opts &o, double tol, void *ws, size_t ws_bytes, cudaStream_t s,
-                   Arena &arena, bool staging_ok) {
+                   CallMemory &arena, bool staging_ok) {
     Plan &pl = P.pl;
     P.o = o;
     P.tol = tol;
@@ -889,7 +865,7 @@ sp2_status run_plan_once(Plan &pl, double tol, const sp2_opts &o, void *ws, size
     sp2_status r = choose_launch(P.pl, o.cta_group, P.grid);
     if (r != SP2_OK) return r;
     *used_cg = (P.pl.path == PATH_TC) ? P.pl.cg : 0;
-    Arena arena(s);
+    CallMemory arena(s);
     arena.fail = (o.test_hook == 2);
     const size_t need = plan_bytes(P.pl);
     if (ws && ws_bytes < need) return SP2_ERR_ARG;
@@ -1219,9 +1195,14 @@ sp2_status sp2_batch_plan_create(int B, const double *const *H, const int *N, co
         }(), 0, &o);
         if (cudaMalloc(&pb->ws, need) != cudaSuccess) {
             cudaGetLastError();
-            return SP2_ERR_NOMEM;
+            pool_release();   // what earlier calls left in the pool
+            if (cudaMalloc(&pb->ws, need) != cudaSuccess) {
+                cudaGetLastError();
+                pb->ws = nullptr;
+                return SP2_ERR_NOMEM;
+            }
         }
-        Arena arena(s);  // unused: every matrix is device-resident
+        CallMemory arena(s);  // unused: every matrix is device-resident
         int want = o.cta_group;
         if (pl.path == PATH_TC && want == 0) {
             const std::string key = tune_key(pl);

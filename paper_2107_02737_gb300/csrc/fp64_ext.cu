@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "device_common.cuh"
+#include "device_pool.h"
 #include "exact.h"
 #include "host_link.h"
 
@@ -97,29 +98,6 @@ int grid_for(size_t work) {
     return g < 1 ? 1 : (int)g;
 }
 
-// Device allocations of one call, freed on every exit path; with `fail` set
-// (sp2_opts.test_hook = 2) every allocation reports failure.
-struct DevBuf {
-    std::vector<void *> p;
-    cudaStream_t s;
-    bool fail = false;
-    explicit DevBuf(cudaStream_t st) : s(st) {}
-    void *get(size_t bytes) {
-        if (fail) return nullptr;
-        void *q = nullptr;
-        if (cudaMallocAsync(&q, bytes ? bytes : 256, s) != cudaSuccess) {
-            cudaGetLastError();
-            return nullptr;
-        }
-        p.push_back(q);
-        return q;
-    }
-    ~DevBuf() {
-        for (void *q : p) cudaFreeAsync(q, s);
-        cudaStreamSynchronize(s);
-    }
-};
-
 #define CKS(x)                        \
     do {                              \
         cudaError_t e_ = (x);         \
@@ -145,7 +123,7 @@ struct CongruenceBufs {
     long long *pscr = nullptr;   // product scratch of the kernel
 };
 
-bool alloc_operand(DevBuf &buf, XsOperand &op, int np, int slices) {
+bool alloc_operand(CallMemory &buf, XsOperand &op, int np, int slices) {
     op.base = (uint16_t *)buf.get((size_t)slices * np * np * 2);
     op.exps = (int *)buf.get((size_t)np * sizeof(int));
     return op.base && op.exps;
@@ -240,7 +218,7 @@ sp2_status run_fp64(const double *H_in, const double *Z_in, int N, double n_occ,
     const unsigned long long timeout_ns = (unsigned long long)(opt.timeout_ms * 1e6);
     const size_t nn = (size_t)N * N;
     const int np = round_up(N, XS_TILE_N);
-    DevBuf buf(s);
+    CallMemory buf(s);
     buf.fail = (opt.test_hook == 2);
     // Inputs on the device: page-locked H from its lower triangle (as every entry
     // point reads it), pageable H and any Z (not symmetric) copied whole.
@@ -427,7 +405,7 @@ extern "C" sp2_status sp2_congruence(const double *Z, const double *M, int N, in
     if (pairs < 1) return SP2_ERR_UNSUPPORTED;
     const int np = round_up(N, XS_TILE_N);
     const size_t nn = (size_t)N * N;
-    DevBuf buf(s);
+    CallMemory buf(s);
     buf.fail = (opt.test_hook == 2);
     CongruenceBufs cb;
     int *d_err = (int *)buf.get(64);

@@ -1,5 +1,5 @@
-"""The tensor-core tile shapes chosen by size (128 x 64, 256 x 128, 256 x 256; compute each element from the same products in the same order, and a layer's
-statistics come from the same partial records whatever tiles it runs in, so a solve is
+"""The tensor-core tile shapes chosen by size (128 x 64, 256 x 128, 256 x 256) compute each
+element from the same products in the same order, and a layer's
 the same bit for bit with every shape: sizes on both sides of each change of shape and
 ragged ones."""
 import pytest
