@@ -439,7 +439,7 @@ int round_tiles(const Plan &pl, int cg, int bn) {
     return pl.mode == MODE_RESPONSE ? 2 * t : t;
 }
 
-// A lone density solve takes narrower tiles where 256 x 256 pair tiles would leave SMs without work: the
+// A lone instance takes narrower tiles where 256 x 256 pair tiles would leave SMs without work: the
 // narrowest whose tiles all run at once.  X is the same with every shape as long as
 // every tile walks K upward, which pair tiles do when an instance has no more of them
 // than the device runs at once.  A tile's K loop is bound by its operand copies (about
@@ -490,7 +490,7 @@ sp2_status choose_launch(Plan &pl, int want, int &grid) {
         // A device constant, so that an instance's tiles walk K the same way in a
         // batch as alone (the accumulation order, and so the bits, follow the tile).
         pl.kwave = std::max(1, grid / pl.cg);
-        if (want == 0 && pl.cg == 2 && pl.dataflow) narrow_tiles(pl, geo, grid);
+        if (want == 0 && pl.cg == 2 && pl.inst.size() == 1) narrow_tiles(pl, geo, grid);
         // No more CTAs than a layer has tiles: the rest would only poll.
         const int tiles = round_tiles(pl, pl.cg, pl.bn);
         pl.flow_blocks = pl.dataflow && pl.bn == TC_BN && tiles > grid / pl.cg;
@@ -810,11 +810,11 @@ sp2_status enqueue(const Prepared &P, cudaStream_t s, cudaEvent_t *ev, bool fres
     // Device hook: CTA 0 withholds its first barrier arrival (test_hook 1, or 3 in a CTA-pair launch).
     rp.test_hook = (P.o.test_hook == 1 || (P.o.test_hook == 3 && pl.path == PATH_TC && pl.cg == 2)) ? 1 : 0;
     if (pl.dataflow) {
-        rp.dataflow = RUN_FLOW;
+        rp.dataflow = pl.flow_blocks ? RUN_FLOW : RUN_WAVE;
         rp.nblk = P.flow_nb;
         rp.tile_done = P.d_tile_done;
         rp.layer_done = (unsigned int *)(P.d_sync + 8);
-        rp.blk_src = pl.flow_blocks ? P.d_blk_src : nullptr;
+        rp.blk_src = P.d_blk_src;
     }
     // A density batch: its own dataflow schedule.
     if (pl.mode == MODE_DENSITY && pl.path == PATH_TC && !pl.dataflow) rp.dataflow = RUN_BATCH;

@@ -40,6 +40,13 @@ __device__ __forceinline__ void ff_add_sq(FF &a, float x, float w) {
     a.c = __fadd_rn(a.c, __fmul_rn(w, e));
 }
 
+// a += x * x
+__device__ __forceinline__ void ff_add_sq1(FF &a, float x) {
+    const float p = __fmul_rn(x, x);
+    ff_add(a, p);
+    a.c = __fadd_rn(a.c, __fmaf_rn(x, x, -p));
+}
+
 // a += b for two compensated pairs (two-sum of the leading parts; the small parts
 // and the sum's rounding error accumulate in a.c).
 __device__ __forceinline__ void ff_add_ff(FF &a, const FF &b) {

@@ -125,10 +125,12 @@ struct InstDesc {
     InstCtl *ctl;
 };
 
-// Schedules of the tensor-core kernel, each its own kernel: rounds ended by a grid
-// barrier (responses, adjoints, layer application), or no barrier between layers
-// for one density solve and for a batch of them.
-enum Schedule { RUN_ROUNDS = 0, RUN_FLOW = 1, RUN_BATCH = 2 };
+// Schedules of the tensor-core kernel, each its own kernel (a layer of a small system is
+// bound by instruction fetch, so no kernel carries another's code): rounds ended by a
+// grid barrier (responses, adjoints, layer application); no barrier between layers
+// for one density solve, whose tiles wait block by block for the previous layer
+// (several waves of tiles) or for all of it (one wave), and for a batch of them.
+enum Schedule { RUN_ROUNDS = 0, RUN_FLOW = 1, RUN_BATCH = 2, RUN_WAVE = 3 };
 
 struct RunParams {
     InstDesc *inst;
@@ -147,8 +149,7 @@ struct RunParams {
     int nblk;                         // dataflow: 256-row blocks of X (round_up(np, 256) / 256)
     unsigned int *tile_done;          // dataflow: per tile, epilogue-warp completions over all layers
     unsigned int *layer_done;         // dataflow: epilogue-warp completions over all layers and tiles
-    const int *blk_src;               // dataflow: [nblk * nblk * 2] tiles writing block (P, Q) of X, -1 none;
-                                      // null: a tile waits for the whole previous layer
+    const int *blk_src;               // dataflow: [nblk * nblk * 2] tiles writing block (P, Q) of X, -1 none
 };
 
 // Host-side launchers (one translation unit each).

@@ -250,14 +250,16 @@ __device__ __forceinline__ bool flow_wait(const RunParams &p, const unsigned int
     return ld_acquire(counter) >= target;
 }
 
-// The eight epilogue warps: one partial record from each warp's compensated pairs, which
+// The eight epilogue warps: one partial record from each warp's compensated pairs (fq: half
+// of ||X||_F^2, an element above the diagonal counting twice), which
 // stay FP32 pairs through the warp and cross-warp sums (FP64 arithmetic is slow on this
 // part); one conversion, written by one thread (epilogue warp 0, lane 0).
 __device__ __forceinline__ void write_record(FF (&red)[EPI_WARPS][4], Part *out, const FF &ft, const FF &fq,
                                              const FF &fw, const FF &fp, int ew, int lane) {
-    FF qw = fq;
+    const FF q = {2.0f * fq.s, 2.0f * fq.c};
+    FF qw = q;
     ff_add_ff(qw, fw);
-    const FF r4[4] = {ff_warp_sum(ft), ff_warp_sum(fq), ff_warp_sum(qw), ff_warp_sum(fp)};
+    const FF r4[4] = {ff_warp_sum(ft), ff_warp_sum(q), ff_warp_sum(qw), ff_warp_sum(fp)};
     if (lane == 0)
 #pragma unroll
         for (int k = 0; k < 4; ++k) red[ew][k] = r4[k];
@@ -285,7 +287,7 @@ __device__ __forceinline__ void flow_record(FF (&red)[EPI_WARPS][4], const InstD
                                          int ew, int lane) {
     const int np = d.np;
     const int2 bt = units[u >> 1];
-    const float *X = d.xf[n & 1];
+    const float *X = xmaster(d, n, false);
     const int rw0 = bt.x * 256 + (u & 1) * 128 + ((ew + 2) & 3) * 32, r = rw0 + lane;
     const int col0 = bt.y * 256 + (ew >> 2) * 128;
     int j0 = 0, j1 = (rw0 < np) ? 128 / EPI_CHUNK : 0;
@@ -313,10 +315,15 @@ __device__ __forceinline__ void flow_record(FF (&red)[EPI_WARPS][4], const InstD
         load(j + 3, u3);
         const int jd = r - (col0 + j * EPI_CHUNK);   // the diagonal's column in the chunk
         float xd = 0.0f;
+        if (col0 + j * EPI_CHUNK > rw0 + 31) {       // strictly above it
 #pragma unroll
-        for (int jj = 0; jj < EPI_CHUNK; ++jj) {
-            ff_add_sq(fq, jj >= jd ? x[jj] : 0.0f, jj == jd ? 1.0f : 2.0f);
-            if (jj == jd) xd = x[jj];
+            for (int jj = 0; jj < EPI_CHUNK; ++jj) ff_add_sq1(fq, x[jj]);
+        } else {
+#pragma unroll
+            for (int jj = 0; jj < EPI_CHUNK; ++jj) {
+                ff_add_sq(fq, jj >= jd ? x[jj] : 0.0f, jj == jd ? 0.5f : 1.0f);
+                if (jj == jd) xd = x[jj];
+            }
         }
         if (jd >= 0 && jd < EPI_CHUNK) {
             ff_add(ft, xd);
@@ -420,10 +427,10 @@ __device__ __noinline__ void flow_owner(RoundCtl &rc, const RunParams &p, int la
 // the others (flow_go by parity: the next decision cannot pass this one's readers, who
 // arrive at its barrier first).  Returns false when the chain stopped or the launch is
 // stopping.
-template <bool NARROW>
+template <bool NARROW, bool ONE_WAVE>
 __device__ __forceinline__ bool flow_decide(RoundCtl &rc, FF (&red)[EPI_WARPS][4], double *sums, const RunParams &p,
                                          int r, int ew, int lane, unsigned int per_layer, const volatile int *abort) {
-    if (!NARROW && !p.blk_src) {
+    if constexpr (!NARROW && ONE_WAVE) {
         // Wide tiles in one wave: one warp does it all while the others wait at the
         // barrier (51.5 against 48.2 us per layer at N = 2304 with the steps below, which
         // win where tiles come in several waves: 121.0 against 122.6 us at N = 4096).
@@ -443,14 +450,14 @@ __device__ __forceinline__ bool flow_decide(RoundCtl &rc, FF (&red)[EPI_WARPS][4
         return rc.flow_go[r & 1] != 0;
     }
     // One thread of a CTA polls (more of them slowed the increments themselves).
-    const bool unit = r > 0 && p.units > 0 && (int)blockIdx.x < p.units;
-    if (r > 0 && (unit || p.units == 0)) {
+    const bool unit = NARROW && r > 0 && (int)blockIdx.x < p.units;
+    if (r > 0 && (unit || !NARROW)) {
         if (ew == 0 && lane == 0 && !flow_wait(p, p.layer_done, per_layer * (unsigned int)r, abort)) sums[4] = 1.0;
         asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32) : "memory");
     }
     // (An aborting launch goes through the same barriers, with whatever X holds.)
     if (unit) flow_record(red, rc.inst[0], p.tiles + rc.inst[0].unit_off, blockIdx.x, r, ew, lane);
-    if (r > 0 && p.units > 0) {
+    if (NARROW && r > 0) {
         if (ew == 0 && lane == 0) {
             if (unit) {
                 __threadfence();
@@ -557,20 +564,18 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
     // that wrote it (and its mirror) have completed.
     int df_round = -1;   // dataflow: layer whose inputs are known to be complete everywhere
     auto produce_tile = [&](const TileWork &w) {
-        // Dataflow: the column block checked last, the one peeked ahead and its counters.
-        int df_kt = -1, df_next = -1;
-        unsigned int df_v[4] = {0u, 0u, 0u, 0u};
-        bool df_ready = SCHED != RUN_FLOW || w.n == 0 || df_round == w.n;
-        if (!df_ready && !p.blk_src) {
-            // One wave of tiles or little more: the layer's tiles end together.
+        if (SCHED == RUN_WAVE && w.n > 0) {
+            // One wave of tiles: the layer's tiles end together.
             if (!flow_wait(p, p.layer_done, (unsigned int)(EPI_WARPS * CG * rc.inst[0].ntiles * w.n), abort)) {
                 tc_abort<CG>(rc, peer_abort);
                 return;
             }
-            df_round = w.n;
-            df_ready = true;
             asm volatile("fence.proxy.async.global;" ::: "memory");
         }
+        // Dataflow: the column block checked last, the one peeked ahead and its counters.
+        int df_kt = -1, df_next = -1;
+        unsigned int df_v[4] = {0u, 0u, 0u, 0u};
+        bool df_ready = SCHED != RUN_FLOW || w.n == 0 || df_round == w.n;
         if (!df_ready) {
             if (ld_relaxed(p.layer_done) >= (unsigned int)(EPI_WARPS * CG * rc.inst[0].ntiles * w.n)) {
                 df_round = w.n;   // every tile of the previous layer is done
@@ -859,7 +864,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
                     }
                     if (stats) {
 #pragma unroll
-                        for (int jj = 0; jj < EPI_CHUNK; ++jj) ff_add_sq(fq, x[jj], 2.0f);
+                        for (int jj = 0; jj < EPI_CHUNK; ++jj) ff_add_sq1(fq, x[jj]);   // weight 2 / 2
                     }
                     // Mirror (c, r): the FP32 master one column per store; the operands two
                     // rows packed per lane, exchanged with the neighbour so that the even
@@ -918,7 +923,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
                         float xd = 0.0f, Pd = 0.0f;
 #pragma unroll
                         for (int jj = 0; jj < EPI_CHUNK; ++jj) {
-                            if (!NARROW) ff_add_sq(fq, jj >= jd ? x[jj] : 0.0f, jj == jd ? 1.0f : 2.0f);
+                            if (!NARROW) ff_add_sq(fq, jj >= jd ? x[jj] : 0.0f, jj == jd ? 0.5f : 1.0f);
                             if (jj == jd) {
                                 xd = x[jj];
                                 Pd = v[jj] * unscale;
@@ -1033,7 +1038,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
                     if (SCHED == RUN_BATCH) {
                         atomicAdd(&d.ctl->flow_done, 1u);
                     } else {
-                        atomicAdd(p.tile_done + w.tile, 1u);
+                        if (SCHED == RUN_FLOW) atomicAdd(p.tile_done + w.tile, 1u);
                         atomicAdd(p.layer_done, 1u);
                     }
                 }
@@ -1136,7 +1141,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
         } else {
             flow_owner<CG>(rc, p, lane, abort);
         }
-    } else if constexpr (SCHED == RUN_FLOW) {
+    } else if constexpr (SCHED == RUN_FLOW || SCHED == RUN_WAVE) {
         // ------------- dataflow schedule (one instance, density mode) -------------
         // No grid barrier between layers.  The producer and the MMA thread run on into
         // the next layer as soon as their own tiles are done (the producer waits per
@@ -1176,7 +1181,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
                 const int g0 = first_tile(r);
                 int2 bt = make_int2(0, 0);
                 if (g0 < ntl) bt = tiles[g0];   // ahead of the wait
-                if (!flow_decide<(BN < 256)>(rc, tl.red, tl.flow_sums, p, r, ew, lane, (unsigned int)(EPI_WARPS * CG * ntl), abort)) {
+                if (!flow_decide<(BN < 256), SCHED == RUN_WAVE>(rc, tl.red, tl.flow_sums, p, r, ew, lane, (unsigned int)(EPI_WARPS * CG * ntl), abort)) {
                     tc_abort<CG>(rc, peer_abort);   // stop rule or error: halt this CTA and its peer
                     break;
                 }
@@ -1206,6 +1211,19 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
                 if (rc.abort) break;
             }
             first = false;
+            // Narrow tiles: the records of the layer just finished, one per CTA, and a
+            // second barrier before they are summed.
+            if (BN < 256 && rc.phase == 0 && rc.active[0] && rc.ran[0]) {
+                if ((int)blockIdx.x < p.units && warp >= 2 && warp < 2 + EPI_WARPS)
+                    flow_record(tl.red, rc.inst[0], p.tiles + rc.inst[0].unit_off, blockIdx.x, rc.layer[0] + 1, ew, lane);
+                __syncthreads();
+                if (threadIdx.x == 0) {
+                    target += gridDim.x;
+                    if (!grid_barrier(p.barrier, target, p.err, p.timeout_ns)) rc.abort = 1;
+                }
+                __syncthreads();
+                if (rc.abort) break;
+            }
             // The epilogue transpose buffers are idle here: use them for the sums.
             reduce_round_partials(rc, p, (double *)epi_T);
             if (p.mode == MODE_ADJOINT) {
@@ -1311,14 +1329,20 @@ const void *tc_kernel_of(int precision) {
                                          : (const void *)k_tc_persistent<SP2_FP16_SPLIT, CG, BN, SCHED>;
 }
 // The tile shapes: 256 x 256 and 128 x 256 with every schedule, 256 x 128 and 128 x 64
-// for a lone density solve.
+// for a lone instance.
 const void *tc_kernel_ptr(int precision, int cg, int bn, int sched) {
     if (sched == RUN_BATCH)
         return cg == 2 ? tc_kernel_of<2, 256, RUN_BATCH>(precision) : tc_kernel_of<1, 256, RUN_BATCH>(precision);
-    if (sched == RUN_ROUNDS)
-        return cg == 2 ? tc_kernel_of<2, 256, RUN_ROUNDS>(precision) : tc_kernel_of<1, 256, RUN_ROUNDS>(precision);
-    if (cg == 2) return bn == 128 ? tc_kernel_of<2, 128, RUN_FLOW>(precision) : tc_kernel_of<2, 256, RUN_FLOW>(precision);
-    return bn == 64 ? tc_kernel_of<1, 64, RUN_FLOW>(precision) : tc_kernel_of<1, 256, RUN_FLOW>(precision);
+    if (sched == RUN_ROUNDS) {
+        if (cg == 2)
+            return bn == 128 ? tc_kernel_of<2, 128, RUN_ROUNDS>(precision) : tc_kernel_of<2, 256, RUN_ROUNDS>(precision);
+        return bn == 64 ? tc_kernel_of<1, 64, RUN_ROUNDS>(precision) : tc_kernel_of<1, 256, RUN_ROUNDS>(precision);
+    }
+    if (sched == RUN_WAVE) {
+        if (cg == 2) return bn == 128 ? tc_kernel_of<2, 128, RUN_WAVE>(precision) : tc_kernel_of<2, 256, RUN_WAVE>(precision);
+        return bn == 64 ? tc_kernel_of<1, 64, RUN_WAVE>(precision) : tc_kernel_of<1, 256, RUN_WAVE>(precision);
+    }
+    return cg == 2 ? tc_kernel_of<2, 256, RUN_FLOW>(precision) : tc_kernel_of<1, 256, RUN_FLOW>(precision);
 }
 
 }  // namespace
@@ -1330,14 +1354,14 @@ static_assert(SMEM_BYTES <= 232448, "dynamic shared memory above the 227 KB a CT
 int tc_grid_size(int cta_group, int bn, int sm_count) {
     const void *fn = nullptr;
     for (int prec : {SP2_FP16_SPLIT, SP2_BF16_SPLIT})
-        for (int sched : {RUN_ROUNDS, RUN_FLOW, RUN_BATCH}) {
+        for (int sched : {RUN_ROUNDS, RUN_FLOW, RUN_BATCH, RUN_WAVE}) {
             fn = tc_kernel_ptr(prec, cta_group, bn, sched);
             if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES) != cudaSuccess) {
                 cudaGetLastError();
                 return 0;
             }
         }
-    fn = tc_kernel_ptr(SP2_FP16_SPLIT, cta_group, bn, RUN_FLOW);
+    fn = tc_kernel_ptr(SP2_FP16_SPLIT, cta_group, bn, RUN_WAVE);
     if (cta_group == 1) {
         int b = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, TC_THREADS, SMEM_BYTES) != cudaSuccess) {
