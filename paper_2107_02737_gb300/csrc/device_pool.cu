@@ -17,7 +17,7 @@ namespace sp2i {
 namespace {
 
 constexpr size_t POOL_KEEP_MAX = (size_t)4 << 30;   // 1.5 % of the device's memory
-constexpr int POOL_WINDOW = 16;
+constexpr int POOL_WINDOW = 12;   // so a large call's memory is back after at most 36 smaller ones
 constexpr int POOL_DEVICES = 64;
 
 struct DevicePool {
