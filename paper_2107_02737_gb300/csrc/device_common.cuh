@@ -562,42 +562,30 @@ __device__ inline void decide_round_parallel(RoundCtl &rc, const RunParams &p, c
     }
 }
 
-// All threads of a CTA, for the FP32 CUDA-core kernel: the same sums with thread k
-// adding entries k, k + blockDim.x, ..., a fixed shuffle tree and a fixed sum over
-// warps, instance after instance.  That kernel runs two CTAs per SM, and there
-// one warp per instance over its 2N^2/128^2 partials costs more than the
-// block-wide pass (measured: +56 ms over a 32-layer chain at N = 8192).  The order
-// again depends only on the instance's partials and the block size.
+// All threads of a CTA, for the FP32 CUDA-core kernel: the sums of the instances still
+// running, one after another.  Half the CTA's lanes take Tr X and half ||X||_F^2 in a
+// fixed stride, then a fixed shuffle tree and a fixed sum over warps.  The order depends
+// only on the instance's partials and the block size.
 __device__ inline void reduce_round_partials_block(const RoundCtl &rc, const RunParams &p, double *sums,
                                                    double *wscratch) {
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5, half = blockDim.x >> 1;
     if (rc.phase == 1) return;
     for (int i = 0; i < p.B; ++i) {
         if (!rc.active[i]) continue;
         const InstDesc &d = p.inst[i];
         const int n = rc.layer[i] + (rc.ran[i] ? 1 : 0);
         const int cnt = (n == 0) ? d.ctl->init_parts : d.parts;
-        const Part *part = d.part[n % 3];
-        double a[4] = {0.0, 0.0, 0.0, 0.0};
+        const double *part = &d.part[n % 3]->t + (tid >= half ? 1 : 0);
+        double a = 0.0;
 #pragma unroll 4
-        for (int k = tid; k < cnt; k += blockDim.x) {
-            const Part v = part[k];
-            a[0] += v.t;
-            a[1] += v.q;
-            a[2] += v.w;
-            a[3] += v.p;
-        }
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-            for (int o = 16; o > 0; o >>= 1) a[c] += __shfl_down_sync(0xffffffffu, a[c], o);
-        if (lane == 0)
-            for (int c = 0; c < 4; ++c) wscratch[wid * 4 + c] = a[c];
+        for (int k = tid % half; k < cnt; k += half) a += __ldcg(part + 4 * (size_t)k);
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+        if (lane == 0) wscratch[wid] = a;
         __syncthreads();
-        if (tid == 0) {
-            double r[4] = {0.0, 0.0, 0.0, 0.0};
-            for (int w = 0; w < nw; ++w)
-                for (int c = 0; c < 4; ++c) r[c] += wscratch[w * 4 + c];
-            for (int c = 0; c < 4; ++c) sums[i * 4 + c] = r[c];
+        if (lane == 0 && wid % (nw / 2) == 0) {
+            for (int w = 1; w < nw / 2; ++w) a += wscratch[wid + w];
+            sums[i * 4 + wid / (nw / 2)] = a;
+            sums[i * 4 + 2 + wid / (nw / 2)] = 0.0;   // no operand offset on this path
         }
         __syncthreads();
     }

@@ -39,7 +39,7 @@ constexpr int max_floats(int a, int b) { return a > b ? a : b; }
 template <int TMAX>
 struct SimtSmem {
     float stage[max_floats(SimtCfg<32>::FLOATS, max_floats(SimtCfg<TMAX >= 64 ? 64 : 32>::FLOATS, SimtCfg<TMAX>::FLOATS))];
-    double red[SIMT_THREADS / 32][2];
+    FF red[SIMT_THREADS / 32][2];
 };
 
 // Two FP32 FMAs in one instruction (each rounded as a scalar FMA): acc = a b + acc.
@@ -285,24 +285,25 @@ __global__ void __launch_bounds__(SIMT_THREADS, TMAX == 128 ? 2 : 4) k_simt_pers
             if (TMAX >= 128 && d.simt_t == 128) simt_tile<TMAX >= 128 ? 128 : 32>(d, n, bt.x, bt.y, flip, alpha, sm.stage, ft, fq);
             else if (TMAX >= 64 && d.simt_t == 64) simt_tile<TMAX >= 64 ? 64 : 32>(d, n, bt.x, bt.y, flip, alpha, sm.stage, ft, fq);
             else simt_tile<32>(d, n, bt.x, bt.y, flip, alpha, sm.stage, ft, fq);
-            // Deterministic block reduction of the tile partials.
-            double t = ff_value(ft), q = ff_value(fq);
-            for (int o = 16; o > 0; o >>= 1) {
-                t += __shfl_down_sync(0xffffffffu, t, o);
-                q += __shfl_down_sync(0xffffffffu, q, o);
-            }
+            // Deterministic block reduction of the tile partials, as compensated pairs up
+            // to one conversion (an FP64 addition takes some 400 cycles here).
+            ft = ff_warp_sum(ft);
+            fq = ff_warp_sum(fq);
             if ((threadIdx.x & 31) == 0) {
-                sm.red[threadIdx.x >> 5][0] = t;
-                sm.red[threadIdx.x >> 5][1] = q;
+                sm.red[threadIdx.x >> 5][0] = ft;
+                sm.red[threadIdx.x >> 5][1] = fq;
             }
             __syncthreads();
             if (threadIdx.x == 0) {
-                Part s;
-                s.t = s.q = s.w = s.p = 0.0;
-                for (int w = 0; w < SIMT_THREADS / 32; ++w) {
-                    s.t += sm.red[w][0];
-                    s.q += sm.red[w][1];
+                FF t = sm.red[0][0], q = sm.red[0][1];
+                for (int w = 1; w < SIMT_THREADS / 32; ++w) {
+                    ff_add_ff(t, sm.red[w][0]);
+                    ff_add_ff(q, sm.red[w][1]);
                 }
+                Part s;
+                s.t = ff_value(t);
+                s.q = ff_value(q);
+                s.w = s.p = 0.0;
                 d.part[(n + 1) % 3][tile] = s;
             }
             __syncthreads();

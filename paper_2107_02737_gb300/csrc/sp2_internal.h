@@ -182,6 +182,7 @@ inline int round_up(int a, int b) { return (a + b - 1) / b * b; }
 //   np 256:  16 /  22 /  49 ( 43)    np 768:   38 /  44 /  95 ( 98)
 //   np 1024: 89 /  54 / 119 (122)    np 1280: 198 / 102 / 144 (150)
 //   np 1664: 375 / 187 / 180 (187)   np 3072: 1776 / 871 / 525 (651)
+// (since then 3 to 5 us less of each layer's fixed cost: 13 at np 256).
 inline int simt_tile_side(int np) { return np <= 768 ? 32 : np <= 1536 ? 64 : 128; }
 
 }  // namespace sp2i

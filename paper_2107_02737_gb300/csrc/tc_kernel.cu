@@ -427,13 +427,13 @@ __device__ __noinline__ void flow_owner(RoundCtl &rc, const RunParams &p, int la
 // the others (flow_go by parity: the next decision cannot pass this one's readers, who
 // arrive at its barrier first).  Returns false when the chain stopped or the launch is
 // stopping.
-template <bool NARROW, bool ONE_WAVE>
+template <bool NARROW>
 __device__ __forceinline__ bool flow_decide(RoundCtl &rc, FF (&red)[EPI_WARPS][4], double *sums, const RunParams &p,
                                          int r, int ew, int lane, unsigned int per_layer, const volatile int *abort) {
-    if constexpr (!NARROW && ONE_WAVE) {
-        // Wide tiles in one wave: one warp does it all while the others wait at the
-        // barrier (51.5 against 48.2 us per layer at N = 2304 with the steps below, which
-        // win where tiles come in several waves: 121.0 against 122.6 us at N = 4096).
+    if constexpr (!NARROW) {
+        // Wide tiles: one warp does it all, beside the next layer's long K loops (48.2
+        // against 51.5 us per layer at N = 2304 with the steps below, no difference in
+        // several waves).
         if (ew == 0) {
             int go = 1;
             if (lane == 0 && r > 0) go = flow_wait(p, p.layer_done, per_layer * (unsigned int)r, abort) ? 1 : 0;
@@ -451,7 +451,7 @@ __device__ __forceinline__ bool flow_decide(RoundCtl &rc, FF (&red)[EPI_WARPS][4
     }
     // One thread of a CTA polls (more of them slowed the increments themselves).
     const bool unit = NARROW && r > 0 && (int)blockIdx.x < p.units;
-    if (r > 0 && (unit || !NARROW)) {
+    if (unit) {
         if (ew == 0 && lane == 0 && !flow_wait(p, p.layer_done, per_layer * (unsigned int)r, abort)) sums[4] = 1.0;
         asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32) : "memory");
     }
@@ -1181,7 +1181,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
                 const int g0 = first_tile(r);
                 int2 bt = make_int2(0, 0);
                 if (g0 < ntl) bt = tiles[g0];   // ahead of the wait
-                if (!flow_decide<(BN < 256), SCHED == RUN_WAVE>(rc, tl.red, tl.flow_sums, p, r, ew, lane, (unsigned int)(EPI_WARPS * CG * ntl), abort)) {
+                if (!flow_decide<(BN < 256)>(rc, tl.red, tl.flow_sums, p, r, ew, lane, (unsigned int)(EPI_WARPS * CG * ntl), abort)) {
                     tc_abort<CG>(rc, peer_abort);   // stop rule or error: halt this CTA and its peer
                     break;
                 }
