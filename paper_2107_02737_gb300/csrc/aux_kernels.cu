@@ -61,51 +61,36 @@ __device__ __forceinline__ double warp_sum_d(double v) {
     return v;
 }
 
-// Block-wide deterministic sum of three doubles; result valid in thread 0.
-__device__ __forceinline__ double3 block_sum3(double a, double b, double c) {
-    __shared__ double sa[AUX_THREADS / 32], sb[AUX_THREADS / 32], sc[AUX_THREADS / 32];
+// Block-wide deterministic sums of K doubles (a fixed tree per warp, then the warps in
+// order, one thread per value: FP64 additions are slow here); valid in every thread.
+template <int K>
+__device__ __forceinline__ void block_sum(double (&v)[K]) {
+    __shared__ double sv[K][AUX_THREADS / 32], out[K];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    a = warp_sum_d(a);
-    b = warp_sum_d(b);
-    c = warp_sum_d(c);
-    if (lane == 0) {
-        sa[w] = a;
-        sb[w] = b;
-        sc[w] = c;
+#pragma unroll
+    for (int c = 0; c < K; ++c) {
+        const double a = warp_sum_d(v[c]);
+        if (lane == 0) sv[c][w] = a;
     }
     __syncthreads();
-    double3 r = make_double3(0.0, 0.0, 0.0);
-    if (threadIdx.x == 0) {
-        for (int k = 0; k < AUX_THREADS / 32; ++k) {
-            r.x += sa[k];
-            r.y += sb[k];
-            r.z += sc[k];
-        }
+    if (threadIdx.x < K) {
+        double r = 0.0;
+        for (int k = 0; k < AUX_THREADS / 32; ++k) r += sv[threadIdx.x][k];
+        out[threadIdx.x] = r;
     }
     __syncthreads();
-    return r;
+#pragma unroll
+    for (int c = 0; c < K; ++c) v[c] = out[c];
 }
-
-// Block-wide deterministic sum of two doubles; result valid in thread 0.
+__device__ __forceinline__ double3 block_sum3(double a, double b, double c) {
+    double v[3] = {a, b, c};
+    block_sum<3>(v);
+    return make_double3(v[0], v[1], v[2]);
+}
 __device__ __forceinline__ double2 block_sum2(double a, double b) {
-    __shared__ double sa[AUX_THREADS / 32], sb[AUX_THREADS / 32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    a = warp_sum_d(a);
-    b = warp_sum_d(b);
-    if (lane == 0) {
-        sa[w] = a;
-        sb[w] = b;
-    }
-    __syncthreads();
-    double2 r = make_double2(0.0, 0.0);
-    if (threadIdx.x == 0) {
-        for (int k = 0; k < AUX_THREADS / 32; ++k) {
-            r.x += sa[k];
-            r.y += sb[k];
-        }
-    }
-    __syncthreads();
-    return r;
+    double v[2] = {a, b};
+    block_sum<2>(v);
+    return make_double2(v[0], v[1]);
 }
 
 // ---------------------------------------------------------------------------
@@ -435,11 +420,33 @@ __global__ void __launch_bounds__(AUX_THREADS, AT_BLOCKS_PER_SM) k_init_x_tc(Ins
     __shared__ uint32_t sp[AT][AT + 1];   // (hi | lo << 16) of the tile, for the mirror
     const InstDesc &d = inst[blockIdx.y];
     const int n = d.n, np = d.np;
-    double emin, emax;
-    resolve_bounds(d, user_bounds != 0, emin, emax);
-    const double delta = emax - emin;
-    const bool degenerate = !(delta > 0.0) || !isfinite(delta) || d.ctl->nonfinite;
-    const double inv = degenerate ? 0.0 : 1.0 / delta;
+    const int nt = np / AT;                          // np is a multiple of 128
+    const long long ntiles = (long long)nt * (nt + 1) / 2;
+    if (blockIdx.x >= ntiles) {   // a small instance of a batch has fewer tiles than blocks
+        if (threadIdx.x == 0) {
+            Part pr;
+            pr.t = pr.q = pr.w = pr.p = 0.0;
+            d.part[0][blockIdx.x] = pr;
+        }
+        return;
+    }
+    // The bounds and their reciprocal by one thread: the FP64 units are shared by an SM's
+    // warps, and every thread of a batch's 34 thousand blocks made a third of the pass.
+    __shared__ double sb[3];
+    __shared__ int sdeg;
+    if (threadIdx.x == 0) {
+        double lo, hi;
+        resolve_bounds(d, user_bounds != 0, lo, hi);
+        const double span = hi - lo;
+        const bool deg = !(span > 0.0) || !isfinite(span) || d.ctl->nonfinite;
+        sb[0] = lo;
+        sb[1] = hi;
+        sb[2] = deg ? 0.0 : 1.0 / span;
+        sdeg = deg ? 1 : 0;
+    }
+    __syncthreads();
+    const double emin = sb[0], emax = sb[1], inv = sb[2];
+    const bool degenerate = sdeg != 0;
     const float inv_hi = (float)inv;                 // 1/delta as a float pair
     const float inv_lo = (float)(inv - (double)inv_hi);
     const float inv_lo24 = inv_hi * 0x1p-24f;       // weight of the 2^24-scaled low part
@@ -452,14 +459,14 @@ __global__ void __launch_bounds__(AUX_THREADS, AT_BLOCKS_PER_SM) k_init_x_tc(Ins
     // diagonal (y = x - 1/2 there) contributes.
     FF ft = {0.f, 0.f}, fq = {0.f, 0.f}, fw = {0.f, 0.f};
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, c0 = 2 * lane;
-    const int nt = np / AT;                          // np is a multiple of 128
-    const long long ntiles = (long long)nt * (nt + 1) / 2;
+    bool any_dg = false;                             // this block has had a diagonal tile
     const bool vec = ((n & 1) == 0) && (((uintptr_t)H & 15) == 0);
     for (long long k = blockIdx.x; k < ntiles; k += gridDim.x) {
         int ti, tj;
         lower_tile(k, ti, tj);
         const int i0 = ti * AT, j0 = tj * AT;
         const bool dg = (ti == tj);
+        any_dg = any_dg || dg;
         double h[AT_RPW][2];
 #pragma unroll
         for (int q = 0; q < AT_RPW; ++q) load_pair(H, n, vec, i0 + w + 8 * q, j0 + c0, h[q][0], h[q][1]);
@@ -521,8 +528,15 @@ __global__ void __launch_bounds__(AUX_THREADS, AT_BLOCKS_PER_SM) k_init_x_tc(Ins
         }
         __syncthreads();
     }
-    ff_add_ff(fw, fq);   // ||Y_0||_F^2
-    double3 s = block_sum3(ff_value(ft), ff_value(fq), ff_value(fw));
+    double3 s;
+    if (any_dg) {
+        ff_add_ff(fw, fq);   // ||Y_0||_F^2
+        s = block_sum3(ff_value(ft), ff_value(fq), ff_value(fw));
+    } else {                 // off the diagonal y = x, and there is no trace
+        double q[1] = {ff_value(fq)};
+        block_sum<1>(q);
+        s = make_double3(0.0, q[0], q[0]);
+    }
     if (threadIdx.x == 0) {
         Part pr;
         pr.t = s.x;
@@ -647,6 +661,10 @@ __global__ void __launch_bounds__(AUX_THREADS, SECOND ? 2 : FIN_BLOCKS_PER_SM) k
     const bool hvec = ((n & 1) == 0) && (((uintptr_t)H & 15) == 0);
     const bool ovec = ((n & 1) == 0) && (((uintptr_t)out & 7) == 0);
     const bool ovec1 = ((n & 1) == 0) && (((uintptr_t)out1 & 7) == 0);
+    if (blockIdx.x >= ntiles) {   // a small instance of a batch, or a small system
+        if (threadIdx.x == 0) d.fin_part[blockIdx.x] = make_double2(0.0, 0.0);
+        return;
+    }
     for (long long k = blockIdx.x; k < ntiles; k += d.fin_blocks) {
         int ti, tj;
         lower_tile(k, ti, tj);

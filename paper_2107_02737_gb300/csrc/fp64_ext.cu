@@ -81,15 +81,19 @@ __global__ void __launch_bounds__(T64) k_energy64(const double *__restrict__ D, 
     if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
-__global__ void k_sum_parts(const double2 *part, int nblocks, double *out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// One block: the partials' sums in a fixed order (a single thread's chain of 512 FP64
+// additions took 55 us).
+__global__ void __launch_bounds__(T64) k_sum_parts(const double2 *part, int nblocks, double *out) {
     double a = 0.0, b = 0.0;
-    for (int k = 0; k < nblocks; ++k) {
+    for (int k = threadIdx.x; k < nblocks; k += T64) {
         a += part[k].x;
         b += part[k].y;
     }
-    out[0] = a;
-    out[1] = b;
+    const double2 s = block_sum2_64(a, b);
+    if (threadIdx.x == 0) {
+        out[0] = s.x;
+        out[1] = s.y;
+    }
 }
 
 int grid_for(size_t work) {
@@ -338,7 +342,7 @@ sp2_status run_fp64(const double *H_in, const double *Z_in, int N, double n_occ,
     // FP64 Tr[D H] (original H) and Tr D.
     const int rb = N < RED_BLOCKS ? N : RED_BLOCKS;
     k_energy64<<<rb, T64, 0, s>>>(Dfin, H, N, part);
-    k_sum_parts<<<1, 32, 0, s>>>(part, rb, d_rec + 4 * (refine_layers + 1));
+    k_sum_parts<<<1, T64, 0, s>>>(part, rb, d_rec + 4 * (refine_layers + 1));
     CKS(cudaGetLastError());
     pe.mark(3, s);
     if (is_device_ptr(D_out)) CKS(cudaMemcpyAsync(D_out, Dfin, nn * 8, cudaMemcpyDeviceToDevice, s));
