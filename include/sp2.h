@@ -135,7 +135,8 @@ typedef struct {
     double eps_min;
     double eps_max;
     int profile;          /* 1 = record per-phase device times into sp2_stats.phase_ms */
-    int cta_group;        /* tensor-core tiles: 0 = choose (default), 1 = one CTA per 128 x 256
+    int cta_group;        /* tensor-core tiles: 0 = choose (default; narrower tiles, of one CTA or a
+                             pair, for a single small system), 1 = one CTA per 128 x 256
                              tile (cooperative launch), 2 = a CTA pair per 256 x 256 tile
                              (M = 256 MMAs; a cluster launch sized to the pairs the device
                              holds at once: work running concurrently on the same GPU can

@@ -13,8 +13,8 @@
 //   warp 0     TMA producer: per K block, the stages of the current sub-pass,
 //              each one A slice (this CTA's 128 rows) and / or one B slice (its
 //              64 of the tile's 128 columns), into a ring of eight 24 KB stages.
-//   warp 1     MMA issuer (even CTA): for every product (A slice s, B slice t)
-//              four K = 16 instructions into the accumulator of level s + t.
+//   warp 1     MMA (even CTA; the warp waits, one elected lane issues): for every
+//              product (A slice s, B slice t) four K = 16 instructions into the accumulator of level s + t.
 //              Tensor memory holds four 128-column accumulators, levels 0..3.
 //              With five or six slices, levels 0..3 are first folded into one
 //              int64 per element (kept in the columns of accumulators 0 and 1)
@@ -756,30 +756,6 @@ __global__ void k_transpose64(const double *__restrict__ M, int n, double *__res
     }
 }
 
-// x 2^k rounded to the nearest integer, ties to even (what __double2ll_rn(x * 2^k) gives),
-// in integer arithmetic: FP64 multiplications and conversions bound the slicing pass
-// otherwise (45 us for a 1800 x 1800 matrix).  Subnormal and non-finite x and results of
-// 2^63 and more go through FP64.
-__device__ __forceinline__ long long fixed_of_double(double x, int k, double sc) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    if ((b << 1) == 0) return 0;
-    const int ex = (int)((b >> 52) & 0x7FF), sh = ex - 1075 + k;
-    if (ex == 0 || ex == 0x7FF || sh > 9) return __double2ll_rn(x * sc);
-    const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-    long long v;
-    if (sh >= 0) {
-        v = (long long)(m << sh);
-    } else if (sh <= -54) {
-        v = 0;   // below one half
-    } else {
-        const int r = -sh;
-        const unsigned long long rem = m & ((1ull << r) - 1), half = 1ull << (r - 1);
-        v = (long long)(m >> r);
-        if (rem > half || (rem == half && (v & 1))) ++v;
-    }
-    return (b >> 63) ? -v : v;
-}
-
 // One warp per row: exponent e with 2^e >= the row's 2-norm, then the slices of
 // the fixed-point value round(x 2^(12 - e + beta (S - 1))) (one bit below the last
 // slice, so that its rounding shift is 1); rows and columns beyond n are zero.
@@ -808,7 +784,7 @@ __global__ void k_xs_slice_rows(const double *__restrict__ M, int n, int np, int
     for (int k = lane; k < np; k += 32) {
         const double x = (row < n && k < n) ? M[(size_t)row * n + k] : 0.0;
         uint16_t a[XS_MAX_SLICES];
-        if (!make_slices(fixed_of_double(x, 12 - e + beta * (slices - 1), sc), slices, beta, beta * (slices - 1) + 1, a)) bad = 1;
+        if (!make_slices(__double2ll_rn(x * sc), slices, beta, beta * (slices - 1) + 1, a)) bad = 1;
 #pragma unroll
         for (int s = 0; s < XS_MAX_SLICES; ++s)
             if (s < slices) sl[(size_t)s * mat + (size_t)row * np + k] = a[s];

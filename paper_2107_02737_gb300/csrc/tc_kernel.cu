@@ -28,9 +28,9 @@
 //               (Y lo, X lo).  The tensor cores' FP32 accumulator truncates once per
 //               MMA instruction; the small cross products of each K block are issued
 //               before its hi x hi product.
-//   warp 1      tcgen05.mma issuer (one thread): M=128, N=256, K=16 per
-//               instruction, FP32 accumulator in TMEM, double-buffered (2 x 256
-//               columns) so the epilogue of tile t overlaps the MMAs of t+1.
+//   warp 1      tcgen05.mma: the warp walks the ring, one elected lane issues (K=16 per
+//               instruction), FP32 accumulator in TMEM, double-buffered so the
+//               epilogue of tile t overlaps the MMAs of t+1.
 //   warps 2..9  epilogue, two warps per SM sub-partition (the epilogue is bound by
 //               instruction latency, so a second warp hides it): warp w reads TMEM
 //               lanes 32 (w mod 4) .. +31 and the tile's column half (w - 2) / 4, in
@@ -38,12 +38,16 @@
 //               operands written for the tile and its mirror (only tiles with rows <=
 //               columns are computed; the direct orientation of a chunk above the
 //               diagonal leaves as two TMA tensor stores), compensated partials of
-//               Tr X and ||X||_F^2 (FP32 pairs, one FP64 record per tile and CTA).
-// Between layers, two schedules.  A single density solve runs without a grid
-// barrier (dataflow): each tile of layer n + 1 starts its K blocks once the tiles
-// of layer n that wrote them have completed, and the epilogue warps alone wait for
-// the whole layer to take its decision.  Batches, responses and adjoints run in
-// rounds ended by a grid barrier, after which every CTA takes the same decisions.
+//               Tr X and ||X||_F^2 (FP32 pairs, one FP64 record per 256 x 256 pair tile
+//               and CTA; with narrower tiles a pass of its own writes the records).
+//   warp 10     the decisions of a batch's instances that this CTA owns.
+// Between layers (Schedule): a density solve runs without a grid barrier.  With
+// several waves of tiles, a tile of layer n + 1 starts its K blocks once the tiles of
+// layer n that wrote them have completed; with one wave, once the layer has.  Only the
+// epilogue needs the layer's sign and offset, so the statistics and the decision run
+// beside the next layer's copies and MMAs.  In a batch each instance advances on its own.
+// Responses, adjoints and layer application run in rounds ended by a grid barrier,
+// after which every CTA takes the same decision.
 // The response / adjoint stream reuses the same machinery with six products per K
 // block: (C + C^T)[i,j] = sum_k X[i,k] Y[j,k] + Y[i,k] X[j,k] for symmetric X and Y.
 #include "device_common.cuh"
