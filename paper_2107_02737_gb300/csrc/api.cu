@@ -444,14 +444,14 @@ int round_tiles(const Plan &pl, int cg, int bn) {
 // every tile walks K upward, which pair tiles do when an instance has no more of them
 // than the device runs at once.  A tile's K loop is bound by its operand copies (about
 // 50 bytes per cycle and SM), so 256 x 128 tiles, whose CTAs share B, beat 128 x 128.
-// Microseconds per layer, 128 x 64 / 256 x 64 / 128 x 128 / 256 x 128 / 256 x 256
-// (before: 256 x 256 only):
-//   N 100:  12.5 / 12.5 / 14.8 / 15.1 / 21.6 (24.6)
-//   N 600:  17.5 / 17.6 / 20.7 / 20.0 / 27.6 (35.0)
-//   N 1280: 24.7 / 26.3 / 27.9 / 28.2 / 36.0 (44.7)
-//   N 1537: 50.4 /  --  / 34.2 / 30.6 / 41.1 (50.6)
-//   N 2048: 59.8 /  --  / 39.2 / 35.6 / 46.6 (56.9)
-//   N 2304: 92.1 /  --  / 69.8 /  --  / 49.3 (61.3)
+// Microseconds per layer, 128 x 64 / 256 x 64 / 128 x 128 / 256 x 128 / 256 x 256, the
+// shapes compared without the statistics pass, then the chosen one as built (and
+// 256 x 256 before there was a choice):
+//   N 100:  12.5 / 12.5 / 14.8 / 15.1 / 21.6   15.8 (24.6)
+//   N 600:  17.5 / 17.6 / 20.7 / 20.0 / 27.6   18.1 (35.0)
+//   N 1537: 50.4 /  --  / 34.2 / 30.6 / 41.1   26.7 (50.6)
+//   N 2048: 59.8 /  --  / 39.2 / 35.6 / 46.6   30.3 (56.9)
+//   N 2304: 92.1 /  --  / 69.8 /  --  / 49.3   48.0 (61.3)
 void narrow_tiles(Plan &pl, const LaunchGeometry &geo, int &grid) {
     for (auto &sp : pl.inst)
         if (ntiles_for(PATH_TC, round_up(sp.n, PAD), 2, TC_BN) > pl.kwave) return;
