@@ -96,6 +96,10 @@ struct TcSmemTail {
     unsigned int consumed;           // MMA thread (even CTA): stages whose copies it has waited for
     FF red[EPI_WARPS][4];            // per epilogue warp: a record's four partials (compensated pairs)
     double flow_sums[5];             // dataflow: the layer's sums; [4] nonzero: a wait gave up
+    struct FlowEntry {               // batch: the decision of a list entry's layer, for the epilogue warps
+        int go, flip;
+        float cf, alpha;
+    } entry[2];
     RoundCtl rc;
     InstDesc desc;                   // a lone instance's descriptor (global loads of it would miss L1
                                      // after every acquire)
@@ -1116,19 +1120,26 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
                     }
                 }
         } else if (warp < 2 + EPI_WARPS) {
+            // One thread waits for a list entry's decision and one barrier hands it to the
+            // eight warps, so that they take the tile or leave together: epilogue_tile has
+            // barriers of its own, and warps that each looked for themselves could part
+            // where a decision and the launch's end meet.  Two entries by parity: one is
+            // written again only after the next one's barrier, which its readers precede.
+            unsigned int e = 0;
             for (int r = 0; any; ++r) {
                 any = false;
                 for (int k = nk - 1; k >= 0; --k) {
                     TileWork w = tile_of(round_tile(k), r);
-                    const InstCtl *ctl = rc.inst[w.inst].ctl;
-                    int go = 0;
-                    if (lane == 0) {
-                        go = flow_wait_instance(p, ctl, r, abort);
-                        w.flip = __ldcg(&ctl->flow_flip);
-                        w.cf = __ldcg(&ctl->flow_cf);
-                        w.alpha = __ldcg(&ctl->flow_alpha);
+                    TcSmemTail::FlowEntry &fe = tl.entry[e++ & 1];
+                    if (ew == 0 && lane == 0) {
+                        const InstCtl *ctl = rc.inst[w.inst].ctl;
+                        fe.go = flow_wait_instance(p, ctl, r, abort);
+                        fe.flip = __ldcg(&ctl->flow_flip);
+                        fe.cf = __ldcg(&ctl->flow_cf);
+                        fe.alpha = __ldcg(&ctl->flow_alpha);
                     }
-                    go = __shfl_sync(0xffffffffu, go, 0);
+                    asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32) : "memory");
+                    const int go = fe.go;
                     if (go < 0) {
                         tc_abort<CG>(rc, peer_abort);
                         any = false;
@@ -1136,9 +1147,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
                     }
                     if (go == 0) continue;
                     any = true;
-                    w.flip = __shfl_sync(0xffffffffu, w.flip, 0);
-                    w.cf = __shfl_sync(0xffffffffu, w.cf, 0);
-                    w.alpha = __shfl_sync(0xffffffffu, w.alpha, 0);
+                    w.flip = fe.flip;
+                    w.cf = fe.cf;
+                    w.alpha = fe.alpha;
                     epilogue_tile(w);
                 }
             }

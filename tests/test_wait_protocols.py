@@ -1,0 +1,39 @@
+"""Waits of the persistent kernels, by their source text: how a warp's or a CTA's threads
+come to act on what one of them waited for.  (A fault here would hang or race on the GPU,
+so it is not provoked there.)"""
+import os
+import re
+
+from paper_2107_02737_gb300 import build
+
+
+def source(name):
+    text = open(os.path.join(build.CSRC, name)).read()
+    return re.sub(r"//[^\n]*", "", text)
+
+
+def block(text, start):
+    """The brace block that opens at or after `start`."""
+    i = text.index("{", start)
+    depth = 0
+    for j in range(i, len(text)):
+        depth += {"{": 1, "}": -1}.get(text[j], 0)
+        if depth == 0:
+            return text[i:j + 1]
+    raise AssertionError("unbalanced braces")
+
+
+def test_batch_epilogue_warps_take_a_decision_together():
+    """The eight epilogue warps meet at named barriers inside a tile's epilogue, so either
+    all of them take a list entry or none does: one thread waits for the entry's decision,
+    and a barrier of all eight lies between that wait and the tile."""
+    batch = block(source("tc_kernel.cu"), source("tc_kernel.cu").index("if constexpr (SCHED == RUN_BATCH) {"))
+    epi = block(batch, batch.index("else if (warp < 2 + EPI_WARPS)"))
+    calls = [m.start() for m in re.finditer(r"flow_wait_instance\(", epi)]
+    assert len(calls) == 1
+    guard = epi.index("if (ew == 0 && lane == 0)")
+    assert guard < calls[0] < guard + len(block(epi, guard)) + len("if (ew == 0 && lane == 0) ")
+    after = epi[calls[0]:epi.index("epilogue_tile(w)")]
+    assert "bar.sync 1" in after
+    # what the warps branch on is what the barrier handed over, nothing of their own
+    assert "*abort" not in after and "__shfl" not in after
