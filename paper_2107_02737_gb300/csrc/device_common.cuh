@@ -167,6 +167,14 @@ __device__ __forceinline__ unsigned int ld_acquire(const unsigned int *p) {
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
+// What lane 0 waited for (an acquire, an mbarrier phase), for its whole warp: a shuffle
+// alone orders no memory, so the other lanes' accesses follow lane 0's wait only through
+// the __syncwarp.
+__device__ __forceinline__ int warp_waited(int lane0) {
+    const int v = __shfl_sync(0xffffffffu, lane0, 0);
+    __syncwarp();
+    return v;
+}
 __device__ __forceinline__ int ld_volatile(const int *p) { return *(const volatile int *)p; }
 
 __device__ __forceinline__ void set_error(int *err, int code) { atomicCAS(err, 0, code); }

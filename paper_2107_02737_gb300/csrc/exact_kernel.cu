@@ -380,7 +380,7 @@ __global__ void __launch_bounds__(XS_THREADS, 1) k_exact_product(const __grid_co
             tile_of(p, g, bi, bj);
             int ok = 1;
             if (lane == 0) ok = mbar_wait(&tl.tfa, (uint32_t)(it & 1), abort, p.timeout_ns, p.err) ? 1 : 0;
-            ok = __shfl_sync(0xffffffffu, ok, 0);
+            ok = warp_waited(ok);
             tc_fence_after();
             const int rw0 = bi * XS_TILE_M + (int)rank * 128 + quarter * 32;   // first row of this warp
             const int r = rw0 + lane;
@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(XS_THREADS, 1) k_exact_product(const __grid_co
                 __syncwarp();
                 if (lane == 0) mbar_arrive_cluster(lead_tea);
                 if (lane == 0 && ok) ok = mbar_wait(&tl.tfb, (uint32_t)(it & 1), abort, p.timeout_ns, p.err) ? 1 : 0;
-                ok = __shfl_sync(0xffffffffu, ok, 0);
+                ok = warp_waited(ok);
                 tc_fence_after();
             }
             // The exact integer products of this warp's chunks, from tensor memory to

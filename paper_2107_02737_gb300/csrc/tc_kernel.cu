@@ -395,7 +395,7 @@ __device__ __noinline__ void flow_owner(RoundCtl &rc, const RunParams &p, int la
                 const unsigned int target = (unsigned int)(EPI_WARPS * CG * rc.inst[i].ntiles) * (unsigned int)n;
                 ready = (ld_relaxed(&ctl->flow_done) >= target && ld_acquire(&ctl->flow_done) >= target) ? 1 : 0;
             }
-            if (!__shfl_sync(0xffffffffu, ready, 0)) continue;
+            if (!warp_waited(ready)) continue;
             double sums[4] = {0.0, 0.0, 0.0, 0.0};
             if (rc.active[i]) sum_layer_partials(rc.inst[i], n, lane, sums);
             int go = 0;
@@ -445,7 +445,7 @@ __device__ __forceinline__ bool flow_decide(RoundCtl &rc, FF (&red)[EPI_WARPS][4
         if (ew == 0) {
             int go = 1;
             if (lane == 0 && r > 0) go = flow_wait(p, p.layer_done, per_layer * (unsigned int)r, abort) ? 1 : 0;
-            go = __shfl_sync(0xffffffffu, go, 0);
+            go = warp_waited(go);
             double a[4];
             if (go) sum_layer_partials(rc.inst[0], r, lane, a);
             if (lane == 0) {
@@ -815,7 +815,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
         }
         int ok = 1;
         if (lane == 0) ok = mbar_wait(&tl.tfull[acc], acc_phase, abort, p.timeout_ns, p.err) ? 1 : 0;
-        ok = __shfl_sync(0xffffffffu, ok, 0);
+        ok = warp_waited(ok);
         tc_fence_after();
         if (ok) {
 #pragma unroll 1
@@ -1107,7 +1107,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
                         const TileWork w = tile_of(round_tile(k), r);
                         int go = 0;
                         if (lane == 0) go = flow_wait_instance(p, rc.inst[w.inst].ctl, r, abort);
-                        go = __shfl_sync(0xffffffffu, go, 0);
+                        go = warp_waited(go);
                         if (go < 0) tc_abort<CG>(rc, peer_abort);
                         if (go > 0) {
                             any = true;

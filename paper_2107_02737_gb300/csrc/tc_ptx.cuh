@@ -84,7 +84,7 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity, c
                                                unsigned long long timeout_ns, int *err) {
     int ok = 1;
     if (!mbar_try_wait(bar, parity) && (threadIdx.x & 31) == 0) ok = mbar_wait(bar, parity, abort, timeout_ns, err) ? 1 : 0;
-    return __shfl_sync(0xffffffffu, ok, 0) != 0;
+    return warp_waited(ok) != 0;
 }
 
 // K-major operand in the 128-byte swizzle layout written by TMA: rows of 128 B,

@@ -37,3 +37,21 @@ def test_batch_epilogue_warps_take_a_decision_together():
     assert "bar.sync 1" in after
     # what the warps branch on is what the barrier handed over, nothing of their own
     assert "*abort" not in after and "__shfl" not in after
+
+
+def test_a_warp_acts_on_lane_0s_wait_only_after_a_warp_barrier():
+    """A shuffle hands a value on but orders no memory: where the value is what lane 0
+    waited for, it goes through warp_waited, which adds the __syncwarp."""
+    waits = r"mbar_wait|flow_wait|flow_wait_instance|ld_acquire"
+    seen = 0
+    for name in ("tc_ptx.cuh", "tc_kernel.cu", "exact_kernel.cu", "simt_kernel.cu"):
+        text = source(name)
+        for m in re.finditer(r"(__shfl_sync\(0xffffffffu, (\w+), 0\)|warp_waited\((\w+)\))", text):
+            var = m.group(2) or m.group(3)
+            assigned = re.findall(r"\b%s = ([^;]*);" % var, text[:m.start()])
+            if assigned and re.search(r"\b(%s)\(" % waits, assigned[-1]):
+                seen += 1
+                assert m.group(3), f"{name}: {assigned[-1]}"
+    assert seen >= 7
+    helper = block(source("device_common.cuh"), source("device_common.cuh").index("int warp_waited(int lane0)"))
+    assert helper.index("__shfl_sync") < helper.index("__syncwarp")
