@@ -134,6 +134,7 @@ struct TileWork {
 template <int CG>
 __device__ __forceinline__ void tc_abort(RoundCtl &rc, uint32_t peer_abort) {
     rc.abort = 1;
+    if (CG == 2) asm volatile("fence.acq_rel.cluster;" ::: "memory");   // after what this CTA has seen
     if (CG == 2) asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(peer_abort), "r"(1) : "memory");
 }
 
@@ -247,7 +248,13 @@ __device__ __forceinline__ bool flow_wait(const RunParams &p, const unsigned int
         const unsigned long long t0 = global_ns();
         for (int i = 0; ld_relaxed(counter) < target; ++i) {
             if ((i & 31) != 31) continue;   // the clock and the flags now and then
-            if (*abort || ld_volatile(p.err) != 0) return false;
+            if (*abort || ld_volatile(p.err) != 0) {
+                // One more look: the other CTA of a pair ends this one once it has seen the
+                // chain's last layer complete, and this one (as CTA 0 it has that decision
+                // to write down) may not have looked since.
+                asm volatile("fence.acq_rel.cluster;" ::: "memory");
+                break;
+            }
             if (global_ns() - t0 > p.timeout_ns) {
                 set_error(p.err, SP2_ERR_TIMEOUT);
                 return false;

@@ -55,3 +55,15 @@ def test_a_warp_acts_on_lane_0s_wait_only_after_a_warp_barrier():
     assert seen >= 7
     helper = block(source("device_common.cuh"), source("device_common.cuh").index("int warp_waited(int lane0)"))
     assert helper.index("__shfl_sync") < helper.index("__syncwarp")
+
+
+def test_a_stopped_wait_looks_at_its_counter_once_more():
+    """The CTA of a pair that first sees the last layer complete ends the other one, which
+    must not take that for a failure of its own wait: CTA 0 writes the last decision."""
+    text = source("tc_kernel.cu")
+    body = block(text, text.index("bool flow_wait(const RunParams &p, const unsigned int *counter"))
+    stop = block(body, body.index("if (*abort || ld_volatile(p.err) != 0)"))
+    assert "return" not in stop and "fence.acq_rel.cluster" in stop and "break" in stop
+    assert body.rstrip().endswith("return ld_acquire(counter) >= target;\n}")
+    halt = block(text, text.index("void tc_abort(RoundCtl &rc"))
+    assert halt.index("fence.acq_rel.cluster") < halt.index("st.shared::cluster")
