@@ -29,8 +29,9 @@ struct SimtCfg {
     static constexpr int TM = T / 8, TN = T / 16;       // 16 x 8, 8 x 4, 4 x 2
     static constexpr int CW = TN < 4 ? TN : 4;          // adjacent columns per thread
     static constexpr int LDS = T + 4;                   // padded smem row (floats), keeps 16-byte alignment
-    static constexpr int KPT = BK * T / SIMT_THREADS;   // K elements of one row a thread stages: 16, 8, 4
+    static constexpr int KPT = BK * T / SIMT_THREADS;   // K elements of one row a thread stages: 8, 8, 4
     static constexpr int FLOATS = 2 * 2 * BK * LDS;     // A and B, double-buffered
+    static constexpr int LEAVES = T * T / 64;           // 4 x 16 blocks of the tile (tile_sums)
 };
 
 constexpr int max_floats(int a, int b) { return a > b ? a : b; }
@@ -39,7 +40,8 @@ constexpr int max_floats(int a, int b) { return a > b ? a : b; }
 template <int TMAX>
 struct SimtSmem {
     float stage[max_floats(SimtCfg<32>::FLOATS, max_floats(SimtCfg<TMAX >= 64 ? 64 : 32>::FLOATS, SimtCfg<TMAX>::FLOATS))];
-    FF red[SIMT_THREADS / 32][2];
+    FF leaf[SimtCfg<TMAX>::LEAVES];   // ||X||_F^2 of the tile's 4 x 16 blocks
+    FF leaf_t[TMAX / 4];              // Tr X of a diagonal tile's 4 x 4 blocks
 };
 
 // Two FP32 FMAs in one instruction (each rounded as a scalar FMA): acc = a b + acc.
@@ -153,7 +155,79 @@ __device__ __forceinline__ void simt_tile_mma(const float *X, int np, int n, int
     }
 }
 
-// SP2 update of one tile, mirror store and FP64 partials.
+// Place of a 4 x 16 block in the tree of a tile's sums: bit 0 its column half of a 32 x 32
+// block, bits 1..3 its row there, then the 32 x 32 block: column, row of a 64 x 64 one,
+// and that one's column, row.
+__device__ __forceinline__ int leaf_index(int row4, int col16) {
+    return (col16 & 1) | ((row4 & 7) << 1) | ((col16 & 2) << 3) | ((row4 & 8) << 2) | ((col16 & 4) << 4) |
+           ((row4 & 16) << 3);
+}
+
+// The whole CTA, after the tile has been stored: Tr X and ||X||_F^2 of its 4 x 16 blocks.  A
+// thread adds 4 x 2 elements at a time as a compensated FP32 pair, a fixed tree makes a
+// block's pair of eight of those, and everything above a block is FP64 (tile_sum).  (One
+// chain over the up to 128 elements a thread computes made ||X||_F^2 2.7e-15 off at
+// N = 3000; blocks of 64 leave 5e-16.)  The elements come back from L2 rather than out of the
+// epilogue's registers, and in a loop that is not unrolled: either of those had the K loop,
+// whose accumulators fill the register file, compiled worse.
+template <int T>
+__device__ __forceinline__ void tile_blocks(const float *X, int np, int r0, int c0, FF *leaf, FF *leaf_t) {
+    constexpr int W = T / 4, UNITS = W * W;   // 4 x 4 units, whole warps of them
+#pragma unroll 1
+    for (int u = threadIdx.x; u < UNITS; u += SIMT_THREADS) {
+        const int row4 = u / W, col4 = u % W, r = r0 + 4 * row4, c = c0 + 4 * col4;
+        float x[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float4 v = r <= c ? __ldcg((const float4 *)(X + (size_t)(r + i) * np + c)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            x[i][0] = v.x;
+            x[i][1] = v.y;
+            x[i][2] = v.z;
+            x[i][3] = v.w;
+        }
+        FF e[2] = {{0.f, 0.f}, {0.f, 0.f}};
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int i = 0; i < 4; ++i)   // an element above the diagonal counts twice
+                ff_add_sq(e[q / 2], x[i][q], (r < c || i < q) ? 2.0f : i == q ? 1.0f : 0.0f);
+        ff_add_ff(e[0], e[1]);
+#pragma unroll
+        for (int o = 1; o < 4; o *= 2) {
+            FF b;
+            b.s = __shfl_down_sync(0xffffffffu, e[0].s, o);
+            b.c = __shfl_down_sync(0xffffffffu, e[0].c, o);
+            ff_add_ff(e[0], b);
+        }
+        if ((col4 & 3) == 0) leaf[leaf_index(row4, col4 >> 2)] = e[0];
+        if (r == c) {
+            FF t = {x[0][0], 0.f}, b = {x[2][2], 0.f};
+            ff_add(t, x[1][1]);
+            ff_add(b, x[3][3]);
+            ff_add_ff(t, b);
+            leaf_t[row4] = t;
+        }
+    }
+}
+
+// One warp: the FP64 sum of a tile's N blocks by a binary tree over their places (valid in lane 0).
+template <int N>
+__device__ __forceinline__ double tile_sum(const FF *leaf, int lane) {
+    constexpr int PER = N > 32 ? N / 32 : 1;   // adjacent places of a lane
+    constexpr int LANES = N / PER;
+    double v[PER];
+#pragma unroll
+    for (int k = 0; k < PER; ++k) v[k] = ff_value(leaf[(lane % LANES) * PER + k]);
+#pragma unroll
+    for (int w = 1; w < PER; w *= 2)
+#pragma unroll
+        for (int k = 0; k < PER; k += 2 * w) v[k] += v[k + w];
+#pragma unroll
+    for (int o = 1; o < LANES; o *= 2) v[0] += __shfl_down_sync(0xffffffffu, v[0], o);
+    return v[0];
+}
+
+// SP2 update of one tile and mirror store.
 // X_{n+1} = k2 X^2 + k1 X + k0 I (I on the n real diagonal entries): the plain
 // layer (1, 0, 0) or (-1, 2, 0); the accelerated one T^2 with T = aX + (1 - a) I,
 // (a^2, 2a(1 - a), (1 - a)^2), or 2T - T^2 with T = aX, (-a^2, 2a, 0).  With
@@ -162,8 +236,7 @@ __device__ __forceinline__ void simt_tile_mma(const float *X, int np, int n, int
 template <int T>
 __device__ __forceinline__ void simt_tile_epilogue(const float *Xold, float *Xnew, int np, int n, int r0, int c0,
                                                    int flip, float alpha,
-                                                   const unsigned long long (&acc)[SimtCfg<T>::TM / 2][SimtCfg<T>::TN],
-                                                   FF &ft, FF &fq) {
+                                                   const unsigned long long (&acc)[SimtCfg<T>::TM / 2][SimtCfg<T>::TN]) {
     using C = SimtCfg<T>;
     const int tid = threadIdx.x;
     const float k2 = flip ? -alpha * alpha : alpha * alpha;
@@ -207,11 +280,8 @@ __device__ __forceinline__ void simt_tile_epilogue(const float *Xold, float *Xne
                     else *(float2 *)p = make_float2(v[i][0], v[i][1]);
                 }
 #pragma unroll
-                for (int q = 0; q < C::CW; ++q) {
+                for (int q = 0; q < C::CW; ++q)
                     *(float4 *)(Xnew + (size_t)(cb + q) * np + rb) = make_float4(v[0][q], v[1][q], v[2][q], v[3][q]);
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) ff_add_sq(fq, v[i][q], 2.0f);
-                }
             } else {
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
@@ -220,26 +290,36 @@ __device__ __forceinline__ void simt_tile_epilogue(const float *Xold, float *Xne
                         const int r = rb + i, c = cb + q;
                         if (r > c) continue;
                         Xnew[(size_t)r * np + c] = v[i][q];
-                        if (r < c) {
-                            Xnew[(size_t)c * np + r] = v[i][q];
-                            ff_add_sq(fq, v[i][q], 2.0f);
-                        } else {
-                            ff_add(ft, v[i][q]);
-                            ff_add_sq(fq, v[i][q], 1.0f);
-                        }
+                        if (r < c) Xnew[(size_t)c * np + r] = v[i][q];
                     }
             }
         }
     }
 }
 
+// Tile (bi, bj) of layer n and its record.
 template <int T>
-__device__ __forceinline__ void simt_tile(const InstDesc &d, int n, int bi, int bj, int flip, float alpha,
-                                          float *stage, FF &ft, FF &fq) {
+__device__ __forceinline__ void simt_tile(const InstDesc &d, int n, int bi, int bj, int tile, int flip, float alpha,
+                                          float *stage, FF *leaf_t, FF *leaf_q) {
     const float *X = d.xf[n & 1];
     unsigned long long acc[SimtCfg<T>::TM / 2][SimtCfg<T>::TN];
     simt_tile_mma<T>(X, d.np, d.n, bi * T, bj * T, stage, acc);
-    simt_tile_epilogue<T>(X, d.xf[(n + 1) & 1], d.np, d.n, bi * T, bj * T, flip, alpha, acc, ft, fq);
+    float *Xn = d.xf[(n + 1) & 1];
+    simt_tile_epilogue<T>(X, Xn, d.np, d.n, bi * T, bj * T, flip, alpha, acc);
+    __syncthreads();
+    tile_blocks<T>(Xn, d.np, bi * T, bj * T, leaf_q, leaf_t);
+    // One warp per value, beside the next tile's staging (the blocks' buffer is written
+    // again only after that tile's K loop and its barriers).
+    __syncthreads();
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    Part *out = d.part[(n + 1) % 3] + tile;
+    if (w == 0) {
+        const double q = tile_sum<SimtCfg<T>::LEAVES>(leaf_q, lane);
+        if (lane == 0) out->q = q;
+    } else if (w == 1) {
+        const double t = bi == bj ? tile_sum<T / 4>(leaf_t, lane) : 0.0;
+        if (lane == 0) out->t = t;
+    }
 }
 
 template <int TMAX>
@@ -281,32 +361,10 @@ __global__ void __launch_bounds__(SIMT_THREADS, TMAX == 128 ? 2 : 4) k_simt_pers
             const int2 bt = p.tiles[d.tile_off + tile];
             const int n = rc.layer[i], flip = rc.choice[i] == SP2_CHOICE_FLIP;
             const float alpha = rc.alpha[i];
-            FF ft = {0.f, 0.f}, fq = {0.f, 0.f};
-            if (TMAX >= 128 && d.simt_t == 128) simt_tile<TMAX >= 128 ? 128 : 32>(d, n, bt.x, bt.y, flip, alpha, sm.stage, ft, fq);
-            else if (TMAX >= 64 && d.simt_t == 64) simt_tile<TMAX >= 64 ? 64 : 32>(d, n, bt.x, bt.y, flip, alpha, sm.stage, ft, fq);
-            else simt_tile<32>(d, n, bt.x, bt.y, flip, alpha, sm.stage, ft, fq);
-            // Deterministic block reduction of the tile partials, as compensated pairs up
-            // to one conversion (an FP64 addition takes some 400 cycles here).
-            ft = ff_warp_sum(ft);
-            fq = ff_warp_sum(fq);
-            if ((threadIdx.x & 31) == 0) {
-                sm.red[threadIdx.x >> 5][0] = ft;
-                sm.red[threadIdx.x >> 5][1] = fq;
-            }
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                FF t = sm.red[0][0], q = sm.red[0][1];
-                for (int w = 1; w < SIMT_THREADS / 32; ++w) {
-                    ff_add_ff(t, sm.red[w][0]);
-                    ff_add_ff(q, sm.red[w][1]);
-                }
-                Part s;
-                s.t = ff_value(t);
-                s.q = ff_value(q);
-                s.w = s.p = 0.0;
-                d.part[(n + 1) % 3][tile] = s;
-            }
-            __syncthreads();
+            FF *lt = sm.leaf_t, *lq = sm.leaf;
+            if (TMAX >= 128 && d.simt_t == 128) simt_tile<TMAX >= 128 ? 128 : 32>(d, n, bt.x, bt.y, tile, flip, alpha, sm.stage, lt, lq);
+            else if (TMAX >= 64 && d.simt_t == 64) simt_tile<TMAX >= 64 ? 64 : 32>(d, n, bt.x, bt.y, tile, flip, alpha, sm.stage, lt, lq);
+            else simt_tile<32>(d, n, bt.x, bt.y, tile, flip, alpha, sm.stage, lt, lq);
         }
     }
 }
