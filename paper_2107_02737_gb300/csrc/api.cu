@@ -130,7 +130,7 @@ struct Carver {
     }
 };
 
-// Tile tables: SIMT uses square tiles with bi <= bj; the tensor-core path uses
+// Tile tables: SIMT uses square tiles of side bn with bi <= bj; the tensor-core path uses
 // 128 cg x bn tiles containing at least one element with row <= column.
 // CTA b takes tiles b, b + grid, ..., so each run of `grid` consecutive tiles is
 // in flight together.  Tiles are ordered by 2048 x 2048 super-blocks (column
@@ -138,8 +138,8 @@ struct Carver {
 // reads a compact set of row and column panels and the operand matrices, which
 // are larger than L2, are fetched from HBM about once per run.
 void build_tiles_uncached(int path, int np, int cg, int tbn, std::vector<int2> &t) {
-    const int bm = (path == PATH_SIMT) ? simt_tile_side(np) : TC_BM * cg;
-    const int bn = (path == PATH_SIMT) ? simt_tile_side(np) : tbn;
+    const int bm = (path == PATH_SIMT) ? tbn : TC_BM * cg;
+    const int bn = tbn;
     const int nbi = (np + bm - 1) / bm, nbj = (np + bn - 1) / bn;  // a last pair tile may overhang np
     const int sbi = 2048 / bm, sbj = 2048 / bn;  // tiles per super-block side
     std::vector<std::pair<long long, int2>> keyed;
@@ -171,8 +171,8 @@ void build_tiles(int path, int np, int cg, int tbn, std::vector<int2> &t) {
 
 // Number of tiles of the table above, counted without building it.
 int ntiles_for(int path, int np, int cg, int tbn) {
-    const int bm = (path == PATH_SIMT) ? simt_tile_side(np) : TC_BM * cg;
-    const int bn = (path == PATH_SIMT) ? simt_tile_side(np) : tbn;
+    const int bm = (path == PATH_SIMT) ? tbn : TC_BM * cg;
+    const int bn = tbn;
     const int nbi = (np + bm - 1) / bm, nbj = (np + bn - 1) / bn;
     int count = 0;
     for (int bj = 0; bj < nbj; ++bj) count += std::min(nbi, ((bj + 1) * bn + bm - 1) / bm);
@@ -185,11 +185,10 @@ int init_blocks_host(int np) { return np < INIT_BLOCKS_MAX ? np : INIT_BLOCKS_MA
 struct Plan {
     int mode, path, precision;
     bool dataflow = false;            // see flow_eligible
-    int cg = 1, bn = TC_BN;           // tensor-core tile: CTAs and columns
+    int cg = 1, bn = TC_BN;           // tensor-core tile: CTAs and columns (FP32 path: bn is the tile side)
     int kwave = 1;                    // InstDesc::kwave
     bool narrow = false;              // tiles narrower than the partial records' (see Part)
     bool flow_blocks = false;         // dataflow: waits per block of X, not per layer
-    int simt_tmax = 128;              // FP32 path: largest tile side of the instances
     std::vector<InstSpec> inst;       // non-trivial instances, in launch order
     std::vector<int> slots;           // nslots_x per instance
     std::vector<int> ckpt_s, ckpt_k;  // adjoint checkpoint stride and kept layers (0: every layer kept)
@@ -250,10 +249,12 @@ void adjoint_layout(int lmax, int stride, int &slots, int &s_out, int &k_out) {
 }
 
 // Partial records per layer: one per tile, per CTA of the tile; with narrow tiles those
-// of the 256 x 256 pair tiles.
+// of the 256 x 256 pair tiles; on the FP32 path per quarter of
+// the 128 x 128 blocks (simt_record).
 int parts_for(const Plan &pl, int np) {
+    if (pl.path == PATH_SIMT) return ntiles_for(pl.path, np, 1, 128) * (pl.bn == 32 ? 16 : 4);
     const int cg = pl.narrow ? 2 : pl.cg, bn = pl.narrow ? TC_BN : pl.bn;
-    return ntiles_for(pl.path, np, cg, bn) * (pl.path == PATH_TC ? cg : 1);
+    return ntiles_for(pl.path, np, cg, bn) * cg;
 }
 
 size_t plan_bytes(const Plan &pl, std::vector<size_t> *offsets_unused = nullptr) {
@@ -467,6 +468,44 @@ void narrow_tiles(Plan &pl, const LaunchGeometry &geo, int &grid) {
     }
 }
 
+// FP32 path: side of a launch's square tiles.  Every element is the same chain of FMAs and
+// a layer's sums the same tree whatever the side, so it is chosen for speed alone: small
+// tiles spread a small matrix over the SMs, large ones reuse a staged value more often.
+// The estimate of a layer is the larger of the longest tile's K loop (ns per k of a CTA
+// alone on its SM) and of the fullest SM's work at the rate of a full SM.  Microseconds
+// per layer with sides 32 / 64 / 128 (and with side 128 only, scalar FMAs, before there
+// was a choice):
+//   N 256:  17.7 / 23.5 / 48 ( 54)     N 768:   39 / 50 / 106 (107)
+//   N 900:    99 / 59 / 134 (132)      N 1536: 255 / 120 / 193 (184)
+//   N 1700:  413 / 206 / 198 (209)     N 3000: 1803 / 894 / 539 (665)
+// and per launch of a batch, milliseconds:
+//   64 x N 256: 12.1 / 8.9 / 7.4 (15.4)    16 x N 768:  20.2 / 14.2 / 12.3 (13.5)
+//   64 x N 768: 78.7 / 44.5 / 33.7 (46.8)  16 x N 1536:  147 / 72 / 58 (66)
+int simt_side(const Plan &pl, int sms) {
+    static const struct {
+        int side;
+        double ns_per_k, fma_per_ns;
+    } shape[3] = {{32, 39.0, 54.0}, {64, 47.0, 112.0}, {128, 104.0, 185.0}};
+    int best = 128;
+    double least = 0.0;
+    for (const auto &t : shape) {
+        double tiles = 0.0, work = 0.0;
+        for (auto &sp : pl.inst) {
+            const int np = round_up(sp.n, PAD);
+            const double k = ntiles_for(PATH_SIMT, np, 1, t.side);
+            tiles += k;
+            work += k * np;
+        }
+        const double per_sm = std::ceil(tiles / sms) * (work / tiles);
+        const double ns = std::max(t.ns_per_k * pl.max_np, per_sm * t.side * t.side / t.fma_per_ns);
+        if (least == 0.0 || ns < least) {
+            least = ns;
+            best = t.side;
+        }
+    }
+    return best;
+}
+
 sp2_status choose_launch(Plan &pl, int want, int &grid) {
     LaunchGeometry geo;
     if (!launch_geometry(geo)) return SP2_ERR_CUDA;
@@ -496,12 +535,12 @@ sp2_status choose_launch(Plan &pl, int want, int &grid) {
         pl.flow_blocks = pl.dataflow && pl.bn == TC_BN && tiles > grid / pl.cg;
         if (tiles < grid / pl.cg) grid = std::max(1, tiles) * pl.cg;
     } else {
-        pl.simt_tmax = simt_tile_side(pl.max_np);
-        const int per_sm = geo.simt_per_sm[pl.simt_tmax == 32 ? 0 : pl.simt_tmax == 64 ? 1 : 2];
+        pl.bn = simt_side(pl, di.sm);
+        const int per_sm = geo.simt_per_sm[pl.bn == 32 ? 0 : pl.bn == 64 ? 1 : 2];
         if (per_sm <= 0) return SP2_ERR_UNSUPPORTED;
         // No more CTAs than a round has tiles: the grid barrier costs less.
         int tiles = 0;
-        for (auto &sp : pl.inst) tiles += ntiles_for(PATH_SIMT, round_up(sp.n, PAD), 1, 0);
+        for (auto &sp : pl.inst) tiles += ntiles_for(PATH_SIMT, round_up(sp.n, PAD), 1, pl.bn);
         grid = std::max(1, std::min(per_sm * di.sm, tiles));
     }
     return SP2_OK;
@@ -596,7 +635,6 @@ sp2_status prepare(Prepared &P, const sp2_opts &o, double tol, void *ws, size_t 
         d.nslots_x = pl.slots[i];
         d.part_cap = std::max(d.parts, initb);
         d.fin_blocks = P.fin_blocks;
-        d.simt_t = (pl.path == PATH_SIMT) ? simt_tile_side(np) : 0;
         d.ctl = d_ctl + i;
         for (int k = 0; k < 3; ++k) d.part[k] = (Part *)c.take(sizeof(Part) * d.part_cap);
         if (pl.path == PATH_TC)
@@ -819,7 +857,7 @@ sp2_status enqueue(const Prepared &P, cudaStream_t s, cudaEvent_t *ev, bool fres
     // A density batch: its own dataflow schedule.
     if (pl.mode == MODE_DENSITY && pl.path == PATH_TC && !pl.dataflow) rp.dataflow = RUN_BATCH;
     if (ev) CK(cudaEventRecord(ev[1], s));
-    CK(pl.path == PATH_TC ? launch_tc_persistent(rp, pl.cg, pl.bn, P.grid, s) : launch_simt_persistent(rp, pl.simt_tmax, P.grid, s));
+    CK(pl.path == PATH_TC ? launch_tc_persistent(rp, pl.cg, pl.bn, P.grid, s) : launch_simt_persistent(rp, pl.bn, P.grid, s));
     if (ev) CK(cudaEventRecord(ev[2], s));
     CK(launch_finalize(P.d_inst, B, P.fin_blocks, pl.mode == MODE_APPLY ? MODE_DENSITY : pl.mode, s));
     if (ev) CK(cudaEventRecord(ev[3], s));
@@ -1054,11 +1092,11 @@ size_t bytes_for(int mode, const std::vector<int> &ns, int layers, const sp2_opt
     set_flow(pl);
     // The tile shape is chosen per device at run time.
     size_t most = 0;
-    for (int cg = 1; cg <= 2; ++cg)
-        for (int bn = 64; bn <= TC_BN; bn *= 2) {
+    for (int cg = 1; cg <= (pl.path == PATH_TC ? 2 : 1); ++cg)
+        for (int bn = pl.path == PATH_TC ? 64 : 32; bn <= (pl.path == PATH_TC ? TC_BN : 128); bn *= 2) {
             pl.cg = cg;
             pl.bn = bn;
-            pl.narrow = bn < TC_BN;
+            pl.narrow = pl.path == PATH_TC && bn < TC_BN;
             most = std::max(most, plan_bytes(pl));
         }
     return most;

@@ -570,33 +570,83 @@ __device__ inline void decide_round_parallel(RoundCtl &rc, const RunParams &p, c
     }
 }
 
+// FP32 path: a layer's sums are kept per 64 x 64 quarter of the 128 x 128 blocks of the
+// upper triangle (the blocks column by column, a block's quarters row by row), whatever
+// the side of the tiles.  With tiles of side 64 a record is one tile's, with side 128 a
+// tile writes four, with side 32 four tiles make a quarter, by the binary tree of their
+// sums: SUB records each.  The first record of tile (bi, bj):
+template <int T>
+__device__ __forceinline__ int simt_record(int bi, int bj) {
+    constexpr int S = 128 / T;
+    const int I = bi / S, J = bj / S, u = bi % S, v = bj % S;
+    const int place = (v & 1) | ((u & 1) << 1) | ((v & 2) << 1) | ((u & 2) << 2);
+    return (J * (J + 1) / 2 + I) * (S == 4 ? 16 : 4) + place;
+}
+
+// The records of a layer: all ||X||_F^2, then all Tr X (every CTA reads all of them, so they
+// lie densely; the input layer's are Parts).
+__device__ __forceinline__ double *simt_records(const InstDesc &d, int n, int c) {
+    return (double *)d.part[n % 3] + (c == 0 ? d.parts : 0);
+}
+
+// One value of quarter q of block k from its SUB records; the quarter below the diagonal of
+// a diagonal block, and its tiles below the diagonal, have no record and count as zero.
+template <int SUB>
+__device__ __forceinline__ double simt_quarter(const double *rec, int k, int cnt, int q) {
+    // Block k is a column's last, the diagonal one, if 8 k + 9 is a square.
+    const int root = (int)(sqrtf((float)(8 * k + 9)) + 0.5f);
+    const bool diagonal = root * root == 8 * k + 9;
+    const bool live = k < cnt && !(diagonal && q == 2);
+    const double *r = rec + ((size_t)k * 4 + q) * SUB;
+    if (SUB == 1) return live ? __ldcg(r) : 0.0;
+    double2 a = make_double2(0.0, 0.0), b = a;
+    if (live) {
+        a = __ldcg((const double2 *)r);
+        b = __ldcg((const double2 *)r + 1);
+        if (diagonal && q != 1) b.x = 0.0;
+    }
+    return (a.x + a.y) + (b.x + b.y);
+}
+
 // All threads of a CTA, for the FP32 CUDA-core kernel: the sums of the instances still
-// running, one after another.  Half the CTA's lanes take Tr X and half ||X||_F^2 in a
-// fixed stride, then a fixed shuffle tree and a fixed sum over warps.  The order depends
-// only on the instance's partials and the block size.
-__device__ inline void reduce_round_partials_block(const RoundCtl &rc, const RunParams &p, double *sums,
-                                                   double *wscratch) {
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5, half = blockDim.x >> 1;
-    if (rc.phase == 1) return;
-    for (int i = 0; i < p.B; ++i) {
+// running, one warp per instance and value (Tr X, ||X||_F^2): lane l adds quarter l mod 4
+// of blocks l / 4, l / 4 + 8, ... (of the input layer, one record per lane), then a fixed
+// shuffle tree.  The order depends only on the instance's size, not on the tiles or the
+// batch.  An FP64 addition holds the SM's FP64 units for 19 cycles per warp, so lanes are
+// not spent on trees before the last one.
+template <int SUB>
+__device__ inline void reduce_round_partials_block(const RoundCtl &rc, const RunParams &p, double *sums) {
+    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    for (int task = threadIdx.x >> 5; task < 2 * p.B; task += nw) {
+        const int i = task >> 1, c = task & 1;
         if (!rc.active[i]) continue;
         const InstDesc &d = p.inst[i];
         const int n = rc.layer[i] + (rc.ran[i] ? 1 : 0);
-        const int cnt = (n == 0) ? d.ctl->init_parts : d.parts;
-        const double *part = &d.part[n % 3]->t + (tid >= half ? 1 : 0);
         double a = 0.0;
+        if (n == 0) {
+            const int cnt = d.ctl->init_parts;
+            const double *part = &d.part[0]->t + c;
 #pragma unroll 4
-        for (int k = tid % half; k < cnt; k += half) a += __ldcg(part + 4 * (size_t)k);
-        for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
-        if (lane == 0) wscratch[wid] = a;
-        __syncthreads();
-        if (lane == 0 && wid % (nw / 2) == 0) {
-            for (int w = 1; w < nw / 2; ++w) a += wscratch[wid + w];
-            sums[i * 4 + wid / (nw / 2)] = a;
-            sums[i * 4 + 2 + wid / (nw / 2)] = 0.0;   // no operand offset on this path
+            for (int k = lane; k < cnt; k += 32) a += __ldcg(part + 4 * (size_t)k);
+        } else {
+            constexpr int AHEAD = SUB == 4 ? 3 : 5;   // loads in flight
+            const int nb = d.np / 128, cnt = nb * (nb + 1) / 2;
+            const double *rec = simt_records(d, n, c);
+            for (int k = lane >> 2; k < cnt; k += 8 * AHEAD) {
+                double v[AHEAD];
+#pragma unroll
+                for (int u = 0; u < AHEAD; ++u) v[u] = simt_quarter<SUB>(rec, k + 8 * u, cnt, lane & 3);
+#pragma unroll
+                for (int u = 0; u < AHEAD; ++u) a += v[u];
+            }
         }
-        __syncthreads();
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+        if (lane == 0) {
+            sums[i * 4 + c] = a;
+            sums[i * 4 + 2 + c] = 0.0;   // no operand offset on this path
+        }
     }
+    __syncthreads();
 }
 
 // Map a round-global tile index to (instance, job, tile).

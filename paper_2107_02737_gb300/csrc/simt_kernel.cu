@@ -1,7 +1,7 @@
 // simt_kernel.cu -- the FP32 CUDA-core SP2 chain (the plain-precision comparator).
 //
 // One cooperative persistent launch runs every layer: per round each CTA takes
-// upper-triangle T x T tiles (bi <= bj; T = 32, 64 or 128 by size) of X_{n+1} = X_n^2 or 2 X_n - X_n^2
+// upper-triangle T x T tiles (bi <= bj; T = 32, 64 or 128 by the launch's work) of X_{n+1} = X_n^2 or 2 X_n - X_n^2
 // (or the accelerated layer), computes the tile's product with FP32 FMAs on the
 // centred operand X - I/2 (the B operand is rows of X because X is symmetric),
 // writes the tile and its mirror, and records FP64 partials of
@@ -21,7 +21,7 @@ namespace {
 // TM TN / 4 cycles of the four FMA pipes).  16 x 8 elements per thread (24 cycles
 // against 32) left room that 8 x 8 (16 against 16) did not, packed FMAs free the issue
 // slots for it, and fragments read one k ahead hide its latency with one or two warps
-// per scheduler: N = 3000 from 651 to 525 us per layer (58 to 72 % of the FP32 peak at
+// per scheduler: N = 3000 from 651 to 539 us per layer (58 to 70 % of the FP32 peak at
 // 1.92 GHz over the executed tiles).
 template <int T>
 struct SimtCfg {
@@ -34,14 +34,11 @@ struct SimtCfg {
     static constexpr int LEAVES = T * T / 64;           // 4 x 16 blocks of the tile (tile_sums)
 };
 
-constexpr int max_floats(int a, int b) { return a > b ? a : b; }
-
-// A launch whose largest side is TMAX also runs tiles of the smaller sides.
-template <int TMAX>
+template <int T>
 struct SimtSmem {
-    float stage[max_floats(SimtCfg<32>::FLOATS, max_floats(SimtCfg<TMAX >= 64 ? 64 : 32>::FLOATS, SimtCfg<TMAX>::FLOATS))];
-    FF leaf[SimtCfg<TMAX>::LEAVES];   // ||X||_F^2 of the tile's 4 x 16 blocks
-    FF leaf_t[TMAX / 4];              // Tr X of a diagonal tile's 4 x 4 blocks
+    float stage[SimtCfg<T>::FLOATS];
+    FF leaf[SimtCfg<T>::LEAVES];   // ||X||_F^2 of the tile's 4 x 16 blocks
+    FF leaf_t[T / 4];              // Tr X of a diagonal tile's 4 x 4 blocks
 };
 
 // Two FP32 FMAs in one instruction (each rounded as a scalar FMA): acc = a b + acc.
@@ -150,9 +147,12 @@ __device__ __forceinline__ void simt_tile_mma(const float *X, int np, int n, int
                 }
             }
         }
-        if (kt + 1 < nk) stash(buf ^ 1, kt + 1);
-        __syncthreads();
+        if (kt + 1 < nk) {
+            stash(buf ^ 1, kt + 1);
+            __syncthreads();
+        }
     }
+    __syncthreads();
 }
 
 // Place of a 4 x 16 block in the tree of a tile's sums: bit 0 its column half of a 32 x 32
@@ -167,11 +167,13 @@ __device__ __forceinline__ int leaf_index(int row4, int col16) {
 // thread adds 4 x 2 elements at a time as a compensated FP32 pair, a fixed tree makes a
 // block's pair of eight of those, and everything above a block is FP64 (tile_sum).  (One
 // chain over the up to 128 elements a thread computes made ||X||_F^2 2.7e-15 off at
-// N = 3000; blocks of 64 leave 5e-16.)  The elements come back from L2 rather than out of the
-// epilogue's registers, and in a loop that is not unrolled: either of those had the K loop,
-// whose accumulators fill the register file, compiled worse.
+// N = 3000; blocks of 64 leave 3e-16.)  The elements come back from L2 (5 to 10 thousand
+// cycles a tile of side 128, of the K loop's 400 to 800), out of line and not unrolled:
+// summed in the epilogue's registers, or unrolled there, they had the K loop, whose
+// accumulators fill the register file, compiled worse (N = 3000: 555 to 595 us per layer
+// instead of 539).
 template <int T>
-__device__ __forceinline__ void tile_blocks(const float *X, int np, int r0, int c0, FF *leaf, FF *leaf_t) {
+__device__ __noinline__ void tile_blocks(const float *X, int np, int r0, int c0, FF *leaf, FF *leaf_t) {
     constexpr int W = T / 4, UNITS = W * W;   // 4 x 4 units, whole warps of them
 #pragma unroll 1
     for (int u = threadIdx.x; u < UNITS; u += SIMT_THREADS) {
@@ -210,20 +212,20 @@ __device__ __forceinline__ void tile_blocks(const float *X, int np, int r0, int 
     }
 }
 
-// One warp: the FP64 sum of a tile's N blocks by a binary tree over their places (valid in lane 0).
-template <int N>
+// One warp: the FP64 sums of a tile's N blocks, in G groups of adjacent places, by a binary
+// tree over the places; group g's is valid in lane g 32 / G (all of it below 32 blocks).
+template <int N, int G>
 __device__ __forceinline__ double tile_sum(const FF *leaf, int lane) {
     constexpr int PER = N > 32 ? N / 32 : 1;   // adjacent places of a lane
-    constexpr int LANES = N / PER;
     double v[PER];
 #pragma unroll
-    for (int k = 0; k < PER; ++k) v[k] = ff_value(leaf[(lane % LANES) * PER + k]);
+    for (int k = 0; k < PER; ++k) v[k] = ff_value(leaf[(lane % (N / PER)) * PER + k]);
 #pragma unroll
     for (int w = 1; w < PER; w *= 2)
 #pragma unroll
         for (int k = 0; k < PER; k += 2 * w) v[k] += v[k + w];
 #pragma unroll
-    for (int o = 1; o < LANES; o *= 2) v[0] += __shfl_down_sync(0xffffffffu, v[0], o);
+    for (int o = 1; o < N / PER / G; o *= 2) v[0] += __shfl_down_sync(0xffffffffu, v[0], o);
     return v[0];
 }
 
@@ -299,7 +301,7 @@ __device__ __forceinline__ void simt_tile_epilogue(const float *Xold, float *Xne
 
 // Tile (bi, bj) of layer n and its record.
 template <int T>
-__device__ __forceinline__ void simt_tile(const InstDesc &d, int n, int bi, int bj, int tile, int flip, float alpha,
+__device__ __forceinline__ void simt_tile(const InstDesc &d, int n, int bi, int bj, int flip, float alpha,
                                           float *stage, FF *leaf_t, FF *leaf_q) {
     const float *X = d.xf[n & 1];
     unsigned long long acc[SimtCfg<T>::TM / 2][SimtCfg<T>::TN];
@@ -312,26 +314,31 @@ __device__ __forceinline__ void simt_tile(const InstDesc &d, int n, int bi, int 
     // again only after that tile's K loop and its barriers).
     __syncthreads();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    Part *out = d.part[(n + 1) % 3] + tile;
+    const int rec = simt_record<T>(bi, bj);
+    constexpr int G = T == 128 ? 4 : 1;   // records of a tile, one per 32 / G lanes
     if (w == 0) {
-        const double q = tile_sum<SimtCfg<T>::LEAVES>(leaf_q, lane);
-        if (lane == 0) out->q = q;
+        const double q = tile_sum<SimtCfg<T>::LEAVES, G>(leaf_q, lane);
+        if (lane % (32 / G) == 0) simt_records(d, n + 1, 1)[rec + lane / (32 / G)] = q;
     } else if (w == 1) {
-        const double t = bi == bj ? tile_sum<T / 4>(leaf_t, lane) : 0.0;
-        if (lane == 0) out->t = t;
+        // Only a diagonal tile has a trace; of its four quarters the first (lane 0) and the
+        // last (summed in lane 16, and lane 24's to write).
+        double t = 0.0;
+        if (bi == bj) {
+            t = tile_sum<T / 4, G == 4 ? 2 : 1>(leaf_t, lane);
+            if (G == 4) {
+                t = __shfl_sync(0xffffffffu, t, lane < 16 ? 0 : 16);
+                if (lane == 8 || lane == 16) t = 0.0;
+            }
+        }
+        if (lane % (32 / G) == 0) simt_records(d, n + 1, 0)[rec + lane / (32 / G)] = t;
     }
 }
 
-template <int TMAX>
-__global__ void __launch_bounds__(SIMT_THREADS, TMAX == 128 ? 2 : 4) k_simt_persistent(const __grid_constant__ RunParams p) {
+template <int T>
+__global__ void __launch_bounds__(SIMT_THREADS, T == 128 ? 2 : 4) k_simt_persistent(const __grid_constant__ RunParams p) {
     __shared__ RoundCtl rc;
-    __shared__ __align__(16) SimtSmem<TMAX> sm;
-    static_assert(sizeof(sm.stage) >= sizeof(float) * SimtCfg<TMAX>::FLOATS &&
-                      (TMAX < 64 || sizeof(sm.stage) >= sizeof(float) * SimtCfg<64>::FLOATS) &&
-                      sizeof(sm.stage) >= sizeof(float) * SimtCfg<32>::FLOATS,
-                  "staging of every side the launch runs");
-    static_assert(sizeof(sm.stage) >= (4 * MAX_BATCH + 4 * (SIMT_THREADS / 32)) * sizeof(double),
-                  "round sums reuse the staging buffers");
+    __shared__ __align__(16) SimtSmem<T> sm;
+    static_assert(sizeof(sm.stage) >= 4 * MAX_BATCH * sizeof(double), "round sums reuse the staging buffers");
     if (threadIdx.x == 0) round_ctl_init(rc, p, p.inst);
     __syncthreads();
     unsigned int target = 0;
@@ -350,7 +357,7 @@ __global__ void __launch_bounds__(SIMT_THREADS, TMAX == 128 ? 2 : 4) k_simt_pers
         first = false;
         // The operand staging buffers are idle here: use them for the sums.
         double *sums = (double *)sm.stage;
-        reduce_round_partials_block(rc, p, sums, sums + 4 * MAX_BATCH);
+        reduce_round_partials_block<(T == 32 ? 4 : 1)>(rc, p, sums);
         if (threadIdx.x == 0) decide_round(rc, p, sums);
         __syncthreads();
         if (rc.abort || rc.total == 0) break;
@@ -361,28 +368,25 @@ __global__ void __launch_bounds__(SIMT_THREADS, TMAX == 128 ? 2 : 4) k_simt_pers
             const int2 bt = p.tiles[d.tile_off + tile];
             const int n = rc.layer[i], flip = rc.choice[i] == SP2_CHOICE_FLIP;
             const float alpha = rc.alpha[i];
-            FF *lt = sm.leaf_t, *lq = sm.leaf;
-            if (TMAX >= 128 && d.simt_t == 128) simt_tile<TMAX >= 128 ? 128 : 32>(d, n, bt.x, bt.y, tile, flip, alpha, sm.stage, lt, lq);
-            else if (TMAX >= 64 && d.simt_t == 64) simt_tile<TMAX >= 64 ? 64 : 32>(d, n, bt.x, bt.y, tile, flip, alpha, sm.stage, lt, lq);
-            else simt_tile<32>(d, n, bt.x, bt.y, tile, flip, alpha, sm.stage, lt, lq);
+            simt_tile<T>(d, n, bt.x, bt.y, flip, alpha, sm.stage, sm.leaf_t, sm.leaf);
         }
     }
 }
 
-const void *simt_kernel(int tmax) {
-    return tmax == 128 ? (const void *)k_simt_persistent<128>
-                       : tmax == 64 ? (const void *)k_simt_persistent<64> : (const void *)k_simt_persistent<32>;
+const void *simt_kernel(int side) {
+    return side == 128 ? (const void *)k_simt_persistent<128>
+                       : side == 64 ? (const void *)k_simt_persistent<64> : (const void *)k_simt_persistent<32>;
 }
 
 }  // namespace
 
-int simt_blocks_per_sm(int tmax) {
+int simt_blocks_per_sm(int side) {
     int b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, simt_kernel(tmax), SIMT_THREADS, 0) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, simt_kernel(side), SIMT_THREADS, 0) != cudaSuccess) return 0;
     return b;
 }
 
-cudaError_t launch_simt_persistent(const RunParams &p, int tmax, int grid, cudaStream_t s) {
+cudaError_t launch_simt_persistent(const RunParams &p, int side, int grid, cudaStream_t s) {
     void *args[] = {(void *)&p};
     // Cooperative launch in the attribute form (also capturable in a CUDA graph).
     cudaLaunchConfig_t cfg = {};
@@ -395,7 +399,7 @@ cudaError_t launch_simt_persistent(const RunParams &p, int tmax, int grid, cudaS
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelExC(&cfg, simt_kernel(tmax), args);
+    return cudaLaunchKernelExC(&cfg, simt_kernel(side), args);
 }
 
 }  // namespace sp2i

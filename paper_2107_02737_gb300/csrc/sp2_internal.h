@@ -113,7 +113,6 @@ struct InstDesc {
     Part *part[3];                    // by layer n mod 3 (three deep for the dataflow schedule)
     float *pdiag[2];                  // narrow tiles: diagonal of the raw product, by layer parity
     int part_cap, fin_blocks;
-    int simt_t, pad_simt;             // FP32 path: tile side (simt_tile_side)
     const CUtensorMap *xmap;          // [nslots_x * MAPS_PER_SLOT]: per slot the K segments' loads op0, op1,
                                       // op2 = hi, hi, lo, then the epilogue's stores of hi and lo
     const CUtensorMap *ymap;          // [2 * MAPS_PER_SLOT]
@@ -164,25 +163,14 @@ cudaError_t launch_init_y(InstDesc *inst, int mode, int precision, cudaStream_t 
 int finalize_blocks();
 cudaError_t launch_finalize(InstDesc *inst, int B, int fin_blocks, int mode, cudaStream_t s);
 cudaError_t launch_fill_trivial(float *D, int n, float diag_value, cudaStream_t s);
-// FP32 path: `tmax` is the largest tile side of the launch's instances.
-cudaError_t launch_simt_persistent(const RunParams &p, int tmax, int grid, cudaStream_t s);
+// FP32 path: `side` is the tiles'.
+cudaError_t launch_simt_persistent(const RunParams &p, int side, int grid, cudaStream_t s);
 cudaError_t launch_tc_persistent(const RunParams &p, int cta_group, int bn, int grid, cudaStream_t s);
-int simt_blocks_per_sm(int tmax);
+int simt_blocks_per_sm(int side);
 int tc_grid_size(int cta_group, int bn, int sm_count);
 // Rows of the operand maps' load boxes for tiles of cg CTAs and bn columns.
 inline int tc_box_rows(int cg, int bn) { return bn / cg < 128 ? bn / cg : 128; }
 
 inline int round_up(int a, int b) { return (a + b - 1) / b * b; }
-
-// Side of the FP32 path's square tiles for an np x np instance.  Every element is the
-// same chain of FMAs whatever the side, so it is chosen for speed alone: small tiles
-// spread a small matrix over the SMs, large ones reuse a staged value more often (the
-// inner loop is bound by shared-memory reads below 128).  Microseconds per layer with
-// sides 32 / 64 / 128 (before: 128 only, scalar FMAs):
-//   np 256:  16 /  22 /  49 ( 43)    np 768:   38 /  44 /  95 ( 98)
-//   np 1024: 89 /  54 / 119 (122)    np 1280: 198 / 102 / 144 (150)
-//   np 1664: 375 / 187 / 180 (187)   np 3072: 1776 / 871 / 525 (651)
-// (since then 3 to 5 us less of each layer's fixed cost: 13 at np 256).
-inline int simt_tile_side(int np) { return np <= 768 ? 32 : np <= 1536 ? 64 : 128; }
 
 }  // namespace sp2i
