@@ -4,41 +4,48 @@
 // (its release threshold is zero), and mapping them again took 0.2 ms of a call at
 // N = 600 and 0.9 ms at N = 4096.  The library's own pool keeps what the latest
 // calls needed, at most POOL_KEEP_MAX bytes: after every POOL_WINDOW calls it is trimmed
-// to the largest call of the last two windows, and it is emptied when an allocation
-// fails.  The pool is CUDA's own stream-ordered one, so blocks move between streams
+// to what the calls of the last two windows held at once (PoolWindow), and it is emptied
+// when an allocation fails.  The pool is CUDA's own stream-ordered one, so blocks move between streams
 // and threads only once their last use is ordered before the next.
 #include "device_pool.h"
 
 #include <algorithm>
 #include <mutex>
 
+#include "pool_window.h"
+
 namespace sp2i {
 
 namespace {
 
 constexpr size_t POOL_KEEP_MAX = (size_t)4 << 30;   // 1.5 % of the device's memory
-constexpr int POOL_WINDOW = 12;   // so a large call's memory is back after at most 36 smaller ones
 constexpr int POOL_DEVICES = 64;
 
 struct DevicePool {
     cudaMemPool_t pool = nullptr;
     bool tried = false;
-    int calls = 0;
-    size_t peak[2] = {0, 0};   // largest call of this window and of the one before
+    PoolWindow window;
 };
 std::mutex g_mu;
 DevicePool g_pool[POOL_DEVICES];
+
+// The current device's entry, nullptr where there is none.
+DevicePool *pool_entry(int &dev) {
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= POOL_DEVICES) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return &g_pool[dev];
+}
 
 // The current device's pool, made on first use; nullptr where there is none (the
 // default pool then serves).
 cudaMemPool_t pool_of_device() {
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= POOL_DEVICES) {
-        cudaGetLastError();
-        return nullptr;
-    }
+    DevicePool *entry = pool_entry(dev);
+    if (!entry) return nullptr;
     std::lock_guard<std::mutex> lock(g_mu);
-    DevicePool &p = g_pool[dev];
+    DevicePool &p = *entry;
     if (!p.tried) {
         p.tried = true;
         cudaMemPoolProps props = {};
@@ -56,25 +63,26 @@ cudaMemPool_t pool_of_device() {
     return p.pool;
 }
 
-// One call that held `bytes` has ended.
+// A call under way has taken `bytes`.
+void pool_held(size_t bytes) {
+    int dev = 0;
+    DevicePool *p = pool_entry(dev);
+    if (!p) return;
+    std::lock_guard<std::mutex> lock(g_mu);
+    p->window.held(bytes);
+}
+
+// A call that had taken `bytes` has ended.
 void pool_call_done(size_t bytes) {
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= POOL_DEVICES) {
-        cudaGetLastError();
-        return;
-    }
+    DevicePool *p = pool_entry(dev);
+    if (!p) return;
     cudaMemPool_t pool = nullptr;
     size_t keep = 0;
     {
         std::lock_guard<std::mutex> lock(g_mu);
-        DevicePool &p = g_pool[dev];
-        p.peak[0] = std::max(p.peak[0], bytes);
-        if (++p.calls < POOL_WINDOW) return;
-        pool = p.pool;
-        keep = std::max(p.peak[0], p.peak[1]);
-        p.peak[1] = p.peak[0];
-        p.peak[0] = 0;
-        p.calls = 0;
+        if (!p->window.ended(bytes, keep)) return;
+        pool = p->pool;
     }
     if (pool && cudaMemPoolTrimTo(pool, std::min(keep + keep / 8, POOL_KEEP_MAX)) != cudaSuccess) cudaGetLastError();
 }
@@ -104,6 +112,7 @@ void *CallMemory::get(size_t bytes) {
     }
     ptrs.push_back(q);
     total += bytes;
+    pool_held(bytes);
     return q;
 }
 
