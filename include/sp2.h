@@ -32,13 +32,18 @@
  *    asymmetric H is unspecified but finite.
  *  - `n_occ` must be an integer value in [0, N].  n_occ = 0 gives D = 0 and
  *    n_occ = N gives D = I without layers.
- *  - `workspace` may be NULL, in which case the call allocates device memory
- *    and frees it before returning; otherwise it must be a device pointer of
+ *  - `workspace` may be NULL, in which case the call takes device memory from a
+ *    pool that the library keeps per device (a memory pool of the CUDA runtime,
+ *    made at the first such call) and returns it to the pool before it returns.
+ *    Between calls the pool holds on to what recent calls needed, at most 4 GiB;
+ *    the runtime gives it back when an allocation in this process would fail
+ *    without it, and sp2_release_memory gives it back at once.
+ *    Otherwise `workspace` must be a device pointer of
  *    at least the size the matching *_workspace_bytes function returns,
  *    256-byte aligned.  Host-resident inputs, and pageable host outputs, are
  *    staged in the workspace beyond that size when it is large enough (8 bytes
  *    per FP64 and 4 per FP32 element, each piece rounded up to 256 bytes), else
- *    in memory the call allocates and frees.
+ *    in memory from the pool.
  *  - Calls are stream-ordered on `stream` (a cudaStream_t; NULL = legacy
  *    default stream) and synchronise that stream before returning, because
  *    the status and the statistics are read back to the host.
@@ -333,9 +338,9 @@ sp2_status sp2_apply_layers(const float *X0, int N, const int *choices, int n_la
  *                       chain (and sp2_density_nonorth's first congruence), [1] the
  *                       refinement layers, [2] the back-transformation and the FP64
  *                       Tr[D H], [3] all of it (CUDA events on the call's stream).
- * Allocates device memory for the FP64 and fixed-point matrices (about 50 bytes
- * per element) and for the chain's workspace, all before the first timed phase,
- * and frees it before returning.
+ * Takes device memory for the FP64 and fixed-point matrices (about 50 bytes
+ * per element) and for the chain's workspace from the pool, all before the
+ * first timed phase, and returns it before it returns.
  * Returns SP2_ERR_NOT_CONVERGED also when X leaves [-2^-13, 1 + 2^-13]
  * spectrally during the refinement (its slices could not hold it exactly).
  */
@@ -398,6 +403,10 @@ sp2_status sp2_congruence(const double *Z, const double *M, int N, int side, dou
 #define SP2_NOALLOC_MAX_N 512
 sp2_status sp2_density_noalloc(const double *H, int N, double n_occ, double tol, float *D,
                                sp2_stats *st, const sp2_opts *o, void *stream);
+
+/* Give the memory that the calls' pool of the current device keeps, and no call under
+ * way uses, back to the device.  Later calls take memory from the device again. */
+sp2_status sp2_release_memory(void);
 
 /* Number of streaming multiprocessors and whether the current device runs this
  * library's kernels (compute capability 10.3). */

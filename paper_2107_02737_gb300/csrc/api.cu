@@ -1163,6 +1163,8 @@ sp2_status sp2_device_info(int *sm_count, int *cc_major, int *cc_minor) {
     return (di.major == 10 && di.minor == 3) ? SP2_OK : SP2_ERR_UNSUPPORTED;
 }
 
+sp2_status sp2_release_memory(void) { return pool_release() == cudaSuccess ? SP2_OK : SP2_ERR_CUDA; }
+
 size_t sp2_density_workspace_bytes(int N, const sp2_opts *o) { return bytes_for(MODE_DENSITY, {N}, 0, o); }
 
 size_t sp2_response_workspace_bytes(int N, const sp2_opts *o) { return bytes_for(MODE_RESPONSE, {N}, 0, o); }

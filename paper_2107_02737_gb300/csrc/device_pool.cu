@@ -89,9 +89,18 @@ void pool_call_done(size_t bytes) {
 
 }  // namespace
 
-void pool_release() {
-    cudaMemPool_t pool = pool_of_device();
-    if (pool && cudaMemPoolTrimTo(pool, 0) != cudaSuccess) cudaGetLastError();
+cudaError_t pool_release() {
+    int dev = 0;
+    DevicePool *p = pool_entry(dev);
+    if (!p) return cudaErrorInvalidDevice;
+    cudaMemPool_t pool = nullptr;
+    {
+        std::lock_guard<std::mutex> lock(g_mu);
+        pool = p->pool;
+    }
+    const cudaError_t e = pool ? cudaMemPoolTrimTo(pool, 0) : cudaSuccess;
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
 }
 
 void *CallMemory::get(size_t bytes) {

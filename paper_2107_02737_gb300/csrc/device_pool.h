@@ -24,6 +24,6 @@ struct CallMemory {
 };
 
 // Gives what the current device's pool keeps, and nothing uses, back to the device.
-void pool_release();
+cudaError_t pool_release();
 
 }  // namespace sp2i

@@ -54,7 +54,7 @@ EXPORTS = ["sp2_default_opts", "sp2_status_string", "sp2_device_info", "sp2_dens
            "sp2_density_batched", "sp2_density_batched_workspace_bytes", "sp2_apply_layers",
            "sp2_density_noalloc", "sp2_density_refined", "sp2_density_nonorth", "sp2_batch_plan_create",
            "sp2_batch_plan_launch", "sp2_batch_plan_stats", "sp2_batch_plan_cta_group", "sp2_batch_plan_destroy",
-           "sp2_congruence"]
+           "sp2_congruence", "sp2_release_memory"]
 NOALLOC_MAX_N = 512
 
 _lib = None
@@ -117,6 +117,8 @@ def load() -> ctypes.CDLL:
     lib.sp2_batch_plan_destroy.restype = None
     lib.sp2_congruence.argtypes = [c_p, c_p, c_i, c_i, c_p, P(Opts), c_p]
     lib.sp2_congruence.restype = c_i
+    lib.sp2_release_memory.argtypes = []
+    lib.sp2_release_memory.restype = c_i
     _lib = lib
     return lib
 
@@ -521,6 +523,11 @@ def device_info():
     sm, ma, mi = ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
     s = load().sp2_device_info(ctypes.byref(sm), ctypes.byref(ma), ctypes.byref(mi))
     return s, sm.value, (ma.value, mi.value)
+
+
+def release_memory():
+    """Give the device memory that the library keeps between calls (at most 4 GiB a device) back."""
+    _check(load().sp2_release_memory(), "sp2_release_memory")
 
 
 class DensityMatrix(torch.autograd.Function):
