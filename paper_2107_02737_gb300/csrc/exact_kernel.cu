@@ -47,9 +47,9 @@ constexpr uint32_t XS_A_BYTES = 128 * TC_BK * 2;   // 16 KB: this CTA's 128 rows
 constexpr uint32_t XS_B_BYTES = 64 * TC_BK * 2;    // 8 KB: this CTA's 64 of the tile's 128 columns
 constexpr uint32_t XS_STAGE_BYTES = XS_A_BYTES + XS_B_BYTES;
 
-// Schedule of one tile, fixed at compile time by the slice count S (so that the
-// MMA warp issues without table look-ups).  Sub-pass 0 holds stages (A_s, B_s),
-// s < min(S, 4), and issues every product of levels 0..3 into accumulator l = s + t.
+// Schedule of one tile, fixed at compile time by the slice count S = 4, 5 or 6 (so that
+// the MMA warp issues without table look-ups).  Sub-pass 0 holds stages (A_s, B_s),
+// s < 4, and issues every product of levels 0..3 into accumulator l = s + t.
 // With S >= 5 two more sub-passes (phase B) issue the products of levels 4 and 5 into
 // accumulators 2 and 3:
 //   sub-pass 1: stages (A3, B1), (A4, B2), (A2, B0) [, (A5, -)]
@@ -60,24 +60,25 @@ constexpr uint32_t XS_STAGE_BYTES = XS_A_BYTES + XS_B_BYTES;
 // only with its whole K block came back a copy's latency late.
 struct Prod {
     int a, b, acc;   // stage holding the A slice, stage holding the B slice, accumulator
+    int s, t;        // the slices
 };
 __host__ __device__ constexpr int sched_nst(int S, int sp) {
-    return sp == 0 ? (S < 4 ? S : 4) : sp == 1 ? (S == 6 ? 4 : 3) : (S == 6 ? 3 : 2);
+    return sp == 0 ? 4 : sp == 1 ? (S == 6 ? 4 : 3) : (S == 6 ? 3 : 2);
 }
 __host__ __device__ constexpr int sched_sa(int S, int sp, int st) {
     constexpr int a1[4] = {3, 4, 2, 5}, a2[3] = {1, 0, 2};
-    return sp == 0 ? sched_nst(S, 0) - 1 - st : sp == 1 ? a1[st] : a2[st];
+    return sp == 0 ? 3 - st : sp == 1 ? a1[st] : a2[st];
 }
 __host__ __device__ constexpr int sched_sb(int S, int sp, int st) {
     constexpr int b1[4] = {1, 2, 0, -1}, b2[3] = {4, 3, 5};
-    return sp == 0 ? sched_nst(S, 0) - 1 - st : sp == 1 ? b1[st] : b2[st];
+    return sp == 0 ? 3 - st : sp == 1 ? b1[st] : b2[st];
 }
 __host__ __device__ constexpr int sched_nprod(int S, int sp) {
-    return sp == 0 ? (S >= 4 ? 10 : S == 3 ? 6 : 3) : sp == 1 ? (S == 6 ? 6 : 3) : (S == 6 ? 5 : 2);
+    return sp == 0 ? 10 : sp == 1 ? (S == 6 ? 6 : 3) : (S == 6 ? 5 : 2);
 }
 __host__ __device__ constexpr Prod sched_prod(int S, int sp, int pr) {
     // The products as slices (s, t), highest slices first: level l = s + t.
-    //   sub-pass 0 (four slices; fewer skip the leading ones): accumulator l
+    //   sub-pass 0: accumulator l
     constexpr int s0[10] = {0, 3, 0, 1, 2, 2, 0, 1, 1, 0}, t0[10] = {3, 0, 2, 2, 1, 0, 1, 1, 0, 0};
     //   sub-pass 1: levels 4, 5 into accumulators 2, 3; five slices have level 4 only
     constexpr int s1[6] = {3, 3, 4, 2, 4, 5}, t1[6] = {1, 2, 1, 2, 0, 0};
@@ -85,16 +86,27 @@ __host__ __device__ constexpr Prod sched_prod(int S, int sp, int pr) {
     //   sub-pass 2
     constexpr int s2[5] = {0, 0, 1, 1, 2}, t2[5] = {5, 4, 4, 3, 3};
     constexpr int s25[2] = {0, 1}, t25[2] = {4, 3};
-    const int k = sp == 0 ? pr + 10 - sched_nprod(S, 0) : pr;
-    const int s = sp == 0 ? s0[k] : sp == 1 ? (S == 6 ? s1[k] : s15[k]) : (S == 6 ? s2[k] : s25[k]);
-    const int t = sp == 0 ? t0[k] : sp == 1 ? (S == 6 ? t1[k] : t15[k]) : (S == 6 ? t2[k] : t25[k]);
-    Prod q{0, 0, sp == 0 ? s + t : s + t - 2};
+    const int s = sp == 0 ? s0[pr] : sp == 1 ? (S == 6 ? s1[pr] : s15[pr]) : (S == 6 ? s2[pr] : s25[pr]);
+    const int t = sp == 0 ? t0[pr] : sp == 1 ? (S == 6 ? t1[pr] : t15[pr]) : (S == 6 ? t2[pr] : t25[pr]);
+    Prod q{0, 0, sp == 0 ? s + t : s + t - 2, s, t};
     for (int st = 0; st < sched_nst(S, sp); ++st) {
         if (sched_sa(S, sp, st) == s) q.a = st;
         if (sched_sb(S, sp, st) == t) q.b = st;
     }
     return q;
 }
+// Every product (s, t) of levels s + t < S is issued once, from the stages that hold its slices.
+constexpr bool sched_complete(int S) {
+    int issued[6][6] = {}, total = 0;
+    for (int sp = 0; sp < (S > 4 ? 3 : 1); ++sp)
+        for (int pr = 0; pr < sched_nprod(S, sp); ++pr, ++total) {
+            const Prod q = sched_prod(S, sp, pr);
+            if (q.s + q.t >= S || sched_sa(S, sp, q.a) != q.s || sched_sb(S, sp, q.b) != q.t) return false;
+            if (issued[q.s][q.t]++ != 0) return false;
+        }
+    return total == S * (S + 1) / 2;
+}
+static_assert(sched_complete(4) && sched_complete(5) && sched_complete(6), "schedule of the slice products");
 // The last product of the sub-pass that reads stage st.
 __host__ __device__ constexpr int sched_last(int S, int sp, int st) {
     int last = 0;
