@@ -47,9 +47,9 @@
  *  - Calls are stream-ordered on `stream` (a cudaStream_t; NULL = legacy
  *    default stream) and synchronise that stream before returning, because
  *    the status and the statistics are read back to the host.
- *  - A wait inside a kernel (the grid barrier between layers; in a single
- *    density solve, the wait for the tiles of the previous layer; a pipeline
- *    barrier) that exceeds `timeout_ms` makes the kernel stop and the call
+ *  - A wait inside a kernel (the grid barrier between layers; in a density solve
+ *    on the tensor cores, the wait for the tiles of the previous layer or for an
+ *    instance's decision; a pipeline barrier) that exceeds `timeout_ms` makes the kernel stop and the call
  *    return SP2_ERR_TIMEOUT; no call leaves a kernel spinning.
  *  - Errors never leave partially written output undefined in size: on any
  *    status other than SP2_OK / SP2_ERR_NOT_CONVERGED the contents of the
@@ -131,8 +131,10 @@ typedef struct {
     int max_layers;       /* default 100, at most SP2_MAX_LAYERS_LIMIT */
     double timeout_ms;    /* device wait limit, default 2000 */
     int user_bounds;      /* 0 = Gershgorin bounds (default), 1 = use eps_min / eps_max below */
-    int test_hook;        /* 0 in normal use; 1 = CTA 0 withholds its first grid-barrier arrival, so
-                             the barrier wait must run out (tests the timeout path); 2 = every
+    int test_hook;        /* 0 in normal use; 1 = CTA 0 withholds what the others wait for first (a
+                             grid-barrier arrival; in a density solve on the tensor cores, single or
+                             batched, a tile's completion), so that their waits must run out (tests
+                             the timeout path); 2 = every
                              device allocation the call makes reports failure (host-side
                              injection; tests the SP2_ERR_NOMEM path); 3 = as 1 but in CTA-pair
                              launches only (a pair that never becomes resident; tests the retry

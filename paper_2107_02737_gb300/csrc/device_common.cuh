@@ -312,8 +312,9 @@ __device__ __forceinline__ double sum_layer_value(const InstDesc &d, int n, int 
     double a = 0.0;
 #pragma unroll 4
     for (int k = lane; k < cnt; k += 32) a += __ldcg(part + 4 * (size_t)k);
-    // Steps that would only add the zeros of lanes without an entry are left out: an FP64
-    // addition takes some 400 cycles here.
+    // Steps that would only add the zeros of lanes without an entry are left out: a step
+    // (shuffle and FP64 addition) takes 110 cycles, more where other warps use the SM's FP64
+    // units, which an addition holds for 19 cycles per warp.
     int o = 16;
     while (o >= cnt && o > 1) o >>= 1;
 #pragma unroll 1
@@ -428,8 +429,10 @@ static __device__ __noinline__ int decide_instance(RoundCtl &rc, const RunParams
         double c = 0.0;
         const float a_made = (n == 0) ? 1.0f : rc.alpha[i];
         if (n > 0) {
-            // (wprev - ps) / n, correctly rounded from the rounded reciprocal by one
-            // residual step (Markstein's theorem): three FP64 operations.
+            // (wprev - ps) / n from the rounded reciprocal and one residual step: three FP64
+            // operations, and correctly rounded.  (The first quotient is within 1.5 ulp, its
+            // residual is exact, and the corrected one before its rounding within 2^-51 ulp;
+            // a quotient by n <= 65536 that is not a midpoint is 2^-17 ulp off any.)
             const double dev = rc.wprev[i] - ps, inv = rc.inv_n[i];
             const double g0 = dev * inv;
             const double gam = isfinite(g0) ? fma(fma(-g0, (double)d.n, dev), inv, g0) : g0;

@@ -68,12 +68,12 @@ struct Cfg {
     static constexpr uint32_t A_BYTES = 128 * TC_BK * 2;                   // 16 KB: own 128 rows
     static constexpr uint32_t B_BYTES = (BN / CG) * TC_BK * 2;             // own B rows
     static constexpr uint32_t STAGE_BYTES = A_BYTES + B_BYTES;
-    static constexpr int STAGES = 196608 / STAGE_BYTES;                    // 4, 6, 8 or 9
+    static constexpr int STAGES = 196608 / STAGE_BYTES;                    // 4, 6 or 8
     static constexpr uint32_t TX_BYTES = STAGE_BYTES * CG;               // bytes per stage over the pair
     static constexpr int TILE_M = 128 * CG;                              // output rows per tile
     static constexpr uint32_t TMEM_COLS = 2 * BN;                        // two FP32 accumulators
 };
-constexpr int MAX_STAGES = 9;
+constexpr int MAX_STAGES = 8;
 constexpr int EPI_WARPS = 8;                              // warps 2..9
 constexpr int EPI_CHUNK = 16;                             // accumulator columns per epilogue step
 // Per epilogue warp: the transpose buffer of a chunk (32 x (EPI_CHUNK + 1) words) or
@@ -105,7 +105,7 @@ struct TcSmemTail {
                                      // after every acquire)
 };
 
-constexpr size_t STAGE_AREA = 196608;  // 4 x 48 KB, 6 x 32 KB, 8 x 24 KB or 9 x 20 KB
+constexpr size_t STAGE_AREA = 196608;  // 4 x 48 KB, 6 x 32 KB or 8 x 24 KB
 static_assert(EPI_WARPS * EPI_T_FLOATS * 4 >= 4 * MAX_BATCH * sizeof(double) + MAX_BATCH * sizeof(int),
               "round sums and decisions reuse the epilogue transpose buffers");
 constexpr size_t SMEM_BYTES = 1024 /*alignment slack*/ + STAGE_AREA + (size_t)EPI_WARPS * EPI_T_FLOATS * 4 +
@@ -465,14 +465,14 @@ __device__ __forceinline__ bool flow_decide(RoundCtl &rc, FF (&red)[EPI_WARPS][4
         return rc.flow_go[r & 1] != 0;
     }
     // One thread of a CTA polls (more of them slowed the increments themselves).
-    const bool unit = NARROW && r > 0 && (int)blockIdx.x < p.units;
+    const bool unit = r > 0 && (int)blockIdx.x < p.units;
     if (unit) {
         if (ew == 0 && lane == 0 && !flow_wait(p, p.layer_done, per_layer * (unsigned int)r, abort)) sums[4] = 1.0;
         asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32) : "memory");
     }
     // (An aborting launch goes through the same barriers, with whatever X holds.)
     if (unit) flow_record(red, rc.inst[0], p.tiles + rc.inst[0].unit_off, blockIdx.x, r, ew, lane);
-    if (NARROW && r > 0) {
+    if (r > 0) {
         if (ew == 0 && lane == 0) {
             if (unit) {
                 __threadfence();
@@ -499,6 +499,7 @@ __device__ __forceinline__ bool flow_decide(RoundCtl &rc, FF (&red)[EPI_WARPS][4
 template <int PREC, int CG, int BN, int SCHED>
 __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_constant__ RunParams p) {
     using C = Cfg<CG, BN>;
+    static_assert(C::STAGES <= MAX_STAGES, "ring of stages");
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t *stages = smem;
@@ -1218,7 +1219,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_persistent(const __grid_co
             }
         }
     } else {
-        // --------------- barrier schedule (every other mode and batch) ---------------
+        // --------- barrier schedule (responses, adjoints, layer application) ---------
         unsigned int target = 0;
         bool first = true;
         while (true) {
