@@ -473,8 +473,8 @@ void narrow_tiles(Plan &pl, const LaunchGeometry &geo, int &grid) {
 // tiles spread a small matrix over the SMs, large ones reuse a staged value more often.
 // The estimate of a layer is the larger of the longest tile's K loop (ns per k of a CTA
 // alone on its SM) and of the fullest SM's work at the rate of a full SM.  Microseconds
-// per layer with sides 32 / 64 / 128 (and with side 128 only, scalar FMAs, before there
-// was a choice):
+// per layer (a call's time over its layers) with sides 32 / 64 / 128 (and with side 128
+// only, scalar FMAs, before there was a choice):
 //   N 256:  17.7 / 23.5 / 48 ( 54)     N 768:   39 / 50 / 106 (107)
 //   N 900:    99 / 59 / 134 (132)      N 1536: 255 / 120 / 193 (184)
 //   N 1700:  413 / 206 / 198 (209)     N 3000: 1803 / 894 / 539 (665)

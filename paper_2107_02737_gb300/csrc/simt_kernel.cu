@@ -1,8 +1,8 @@
 // simt_kernel.cu -- the FP32 CUDA-core SP2 chain (the plain-precision comparator).
 //
 // One cooperative persistent launch runs every layer: per round each CTA takes
-// upper-triangle T x T tiles (bi <= bj; T = 32, 64 or 128 by the launch's work) of X_{n+1} = X_n^2 or 2 X_n - X_n^2
-// (or the accelerated layer), computes the tile's product with FP32 FMAs on the
+// upper-triangle T x T tiles (bi <= bj; T = 32, 64 or 128 by the launch's work) of
+// X_{n+1} = X_n^2 or 2 X_n - X_n^2 (or the accelerated layer), computes the tile's product with FP32 FMAs on the
 // centred operand X - I/2 (the B operand is rows of X because X is symmetric),
 // writes the tile and its mirror, and records FP64 partials of
 // Tr X_{n+1} and ||X_{n+1}||_F^2.  A grid barrier ends the round; every CTA then
@@ -12,7 +12,6 @@
 namespace sp2i {
 
 namespace {
-
 
 // Tile side T with 128 threads as 8 (rows) x 16 (columns): a thread owns TM x TN
 // elements, rows in groups of four 32 apart, columns in groups of CW 16 CW apart.
@@ -31,7 +30,7 @@ struct SimtCfg {
     static constexpr int LDS = T + 4;                   // padded smem row (floats), keeps 16-byte alignment
     static constexpr int KPT = BK * T / SIMT_THREADS;   // K elements of one row a thread stages: 8, 8, 4
     static constexpr int FLOATS = 2 * 2 * BK * LDS;     // A and B, double-buffered
-    static constexpr int LEAVES = T * T / 64;           // 4 x 16 blocks of the tile (tile_sums)
+    static constexpr int LEAVES = T * T / 64;           // 4 x 16 blocks of the tile (tile_blocks)
 };
 
 template <int T>

@@ -16,7 +16,7 @@
 //   part[3]     FP64 partials, by layer n mod 3: Tr X, ||X||_F^2, ||Y||_F^2 and Tr P
 //               (see Part).
 //   dataflow schedule (one instance, density mode, tensor cores): three operand
-//               slots; per tile a completion counter (CTAs done, all layers) and a
+//               slots; per tile a completion counter (epilogue warps done, all layers) and a
 //               table of the tiles that write each 256 x 256 block of X.
 // Tensor-core path: the operands are the split of Y = X - I/2 (identity on the
 // first N diagonal entries only), and the true X_n is the stored FP32 X_n plus
@@ -57,12 +57,13 @@ enum Mode { MODE_DENSITY = 0, MODE_RESPONSE = 1, MODE_ADJOINT = 2, MODE_APPLY = 
 // FP64 partial sums written by the input layer and every square: on the tensor-core
 // path one record per 256 x 256 pair tile and CTA (128 x 256 tile where those are used),
 // whatever tiles the layer itself runs in, so that a layer's sums, and with them every
-// bit of the chain, do not depend on the tile shape.
+// bit of the chain, do not depend on the tile shape.  (The FP32 path's layers keep Tr X
+// and ||X||_F^2 densely in the same buffers: simt_records.)
 struct __align__(16) Part {
     double t;   // Tr X (stored X)
     double q;   // ||X||_F^2 (stored X)
-    double w;   // ||Y||_F^2 of the split operand matrix Y the next square multiplies (0 on the FP32 path)
-    double p;   // Tr P, P the raw product of this square (0 on the FP32 path)
+    double w;   // ||Y||_F^2 of the split operand matrix Y the next square multiplies
+    double p;   // Tr P, P the raw product of this square
 };
 
 struct LayerStatDev {
